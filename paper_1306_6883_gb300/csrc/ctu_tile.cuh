@@ -621,7 +621,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
           if constexpr (is_f32<R>())
             div = (su[cR] - su[cL]) * s.idx + dvy * (0.25f * s.idy);
           else
-            div = (su[cR] - su[cL]) / s.dx + dvy / (4.0 * s.dy);
+            div = soft_div(su[cR] - su[cL], s.dx) + soft_div(dvy, 4.0 * s.dy);
           const R av = s.cvisc * M<R>::mx(-div * s.dx, (R)0);
           if constexpr (L::SMEM_U) {
             R uL[4], uR[4], du[4];
@@ -650,7 +650,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
           if constexpr (is_f32<R>())
             div = (sv[cR] - sv[cL]) * s.idy + dux * (0.25f * s.idx);
           else
-            div = (sv[cR] - sv[cL]) / s.dy + dux / (4.0 * s.dx);
+            div = soft_div(sv[cR] - sv[cL], s.dy) + soft_div(dux, 4.0 * s.dx);
           const R av = s.cvisc * M<R>::mx(-div * s.dy, (R)0);
           if constexpr (L::SMEM_U) {
             R uL[4], uR[4], du[4];

@@ -13,6 +13,8 @@
 
 #include <type_traits>
 
+#include "soft_f64.cuh"
+
 namespace hydro {
 
 // Parameters as the kernels see them (plain values, passed by value).
@@ -110,8 +112,8 @@ struct M;
 
 template <>
 struct M<double> {
-  static __device__ __forceinline__ double sq(double x) { return sqrt(x); }
-  static __device__ __forceinline__ double dv(double a, double b) { return a / b; }
+  static __device__ __forceinline__ double sq(double x) { return soft_sqrt(x); }
+  static __device__ __forceinline__ double dv(double a, double b) { return soft_div(a, b); }
   static __device__ __forceinline__ double mn(double a, double b) { return fmin(a, b); }
   static __device__ __forceinline__ double mx(double a, double b) { return fmax(a, b); }
   static __device__ __forceinline__ double ab(double a) { return fabs(a); }
@@ -291,8 +293,8 @@ __device__ __forceinline__ void cons_to_prim(const SP<R>& s, R U0, R U1, R U2, R
       p = s.gm1 * (U3 - ke);
     }
   } else {
-    u = U1 / rho;
-    v = U2 / rho;
+    u = soft_div(U1, rho);
+    v = soft_div(U2, rho);
     const double ke = 0.5 * rho * (u * u + v * v);
     p = s.gm1 * (U3 - ke);
   }
@@ -308,7 +310,7 @@ __device__ __forceinline__ void prim_to_cons(const SP<R>& s, R rho, R u, R v, R 
   if constexpr (is_f32<R>())
     U3 = p * s.igm1 + 0.5f * rho * (u * u + v * v);
   else
-    U3 = p / s.gm1 + 0.5 * rho * (u * u + v * v);
+    U3 = soft_div(p, s.gm1) + 0.5 * rho * (u * u + v * v);
 }
 
 // Pressure of a transversely corrected FP32 face state formed in double (see correct_state): the state's
@@ -418,8 +420,8 @@ __device__ __forceinline__ R flatten_chi(R pm2, R pm1, R pp1, R pp2, R um1, R up
     const float z = M<float>::ab(dp1) * rcpa(M<float>::mx(M<float>::ab(dp2), small_pres));
     chi = 1.0f - (z - z0) * (1.0f / (0.85f - 0.75f));
   } else {
-    R z = M<R>::ab(dp1) / M<R>::mx(M<R>::ab(dp2), small_pres);
-    chi = (R)1 - (z - z0) / (z1 - z0);
+    R z = soft_div(M<R>::ab(dp1), M<R>::mx(M<R>::ab(dp2), small_pres));
+    chi = (R)1 - soft_div(z - z0, z1 - z0);
   }
   chi = chi < (R)0 ? (R)0 : chi;
   chi = chi > (R)1 ? (R)1 : chi;
@@ -449,12 +451,12 @@ __device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], con
     ic2h = 0.5f * ic2;
     cor = c * ir;
   } else {
-    c = sqrt(s.gamma * pres / rho);
+    c = soft_sqrt(soft_div(s.gamma * pres, rho));
     c2 = c * c;
-    roc = (0.5 * rho) / c;
-    ic2h = 0.5 / c2;
-    ic2 = 1.0 / c2;
-    cor = c / rho;
+    roc = soft_div(0.5 * rho, c);
+    ic2h = soft_div(0.5, c2);
+    ic2 = soft_div(1.0, c2);
+    cor = soft_div(c, rho);
   }
   const R lam1 = un - c, lam2 = un, lam4 = un + c;
   const R b1 = -roc * dq[1] + ic2h * dq[3];
@@ -547,8 +549,8 @@ __device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R&
     l = a1 + 0.5f * (a2 - a1) - (d0 - dm) * (1.0f / 6.0f);
     r = a2 + 0.5f * (a3 - a2) - (dp - d0) * (1.0f / 6.0f);
   } else {
-    l = a1 + 0.5 * (a2 - a1) - (d0 - dm) / 6.0;
-    r = a2 + 0.5 * (a3 - a2) - (dp - d0) / 6.0;
+    l = a1 + 0.5 * (a2 - a1) - soft_div(d0 - dm, 6.0);
+    r = a2 + 0.5 * (a3 - a2) - soft_div(dp - d0, 6.0);
   }
   const bool flat = (r - c) * (c - l) <= (R)0;
   const R da = r - l, mid = c - (R)0.5 * (l + r);
@@ -556,9 +558,14 @@ __device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R&
   if constexpr (is_f32<R>())
     d6 = da * da * (1.0f / 6.0f);
   else
-    d6 = da * da / 6.0;
+    d6 = soft_div(da * da, 6.0);
   const bool left_ex = da * mid > d6;
-  const bool right_ex = !left_ex && -(da * da) / (R)6 > da * mid;
+  R d6r;
+  if constexpr (is_f32<R>())
+    d6r = -(da * da) / (R)6;
+  else
+    d6r = soft_div(-(da * da), 6.0);
+  const bool right_ex = !left_ex && d6r > da * mid;
   const R l2 = flat ? c : (left_ex ? (R)3 * c - (R)2 * r : l);
   const R r2 = flat ? c : (right_ex ? (R)3 * c - (R)2 * l : r);
   eL = xi * l2 + ((R)1 - xi) * c;
@@ -588,12 +595,12 @@ __device__ __forceinline__ void trace_ppm(const SP<R>& s, R sigma, const R q[4],
     ic2h = 0.5f * ic2;
     cor = c * ir;
   } else {
-    c = sqrt(s.gamma * pres / rho);
+    c = soft_sqrt(soft_div(s.gamma * pres, rho));
     c2 = c * c;
-    roc = (0.5 * rho) / c;
-    ic2h = 0.5 / c2;
-    ic2 = 1.0 / c2;
-    cor = c / rho;
+    roc = soft_div(0.5 * rho, c);
+    ic2h = soft_div(0.5, c2);
+    ic2 = soft_div(1.0, c2);
+    cor = soft_div(c, rho);
   }
   const R lam1 = un - c, lam2 = un, lam4 = un + c;
   R da[4], a6[4];
@@ -702,7 +709,7 @@ __device__ __forceinline__ void face_flux(const SP<R>& s, R fr, R fu, R fv, R fp
   if constexpr (is_f32<R>())
     rhoE = fp * s.igm1 + 0.5f * fr * (fu * fu + fv * fv);
   else
-    rhoE = fp / s.gm1 + 0.5 * fr * (fu * fu + fv * fv);
+    rhoE = soft_div(fp, s.gm1) + 0.5 * fr * (fu * fu + fv * fv);
   F[0] = fr * fu;
   F[1] = fr * fu * fu + fp;
   F[2] = fr * fu * fv;
@@ -720,36 +727,36 @@ __device__ __forceinline__ void riemann(const SP<double>& s, const double qL[4],
   const double g = s.gamma, g1 = s.g1;
   const double rl = qL[0], ul = qL[1], vl = qL[2], pl = qL[3];
   const double rr = qR[0], ur = qR[1], vr = qR[2], pr = qR[3];
-  const double cl = sqrt(g * pl * rl);
-  const double cr = sqrt(g * pr * rr);
+  const double cl = soft_sqrt(g * pl * rl);
+  const double cr = soft_sqrt(g * pr * rr);
   // stop also once the step's velocity mismatch |dp| (1/Z_L + 1/Z_R) is below tol times the velocity scale
-  const double vscale = fabs(ul) + fabs(ur) + cl / rl + cr / rr;
-  double pst = guess > 0.0 ? guess : (cr * pl + cl * pr + cl * cr * (ul - ur)) / (cl + cr);
+  const double vscale = fabs(ul) + fabs(ur) + soft_div(cl, rl) + soft_div(cr, rr);
+  double pst = guess > 0.0 ? guess : soft_div(cr * pl + cl * pr + cl * cr * (ul - ur), cl + cr);
   pst = pst < s.small_pres ? s.small_pres : pst;
   int it = 0;
   bool ok = false;
   while (it < s.maxiter) {
-    double wl = cl * sqrt(1.0 + g1 * (pst / pl - 1.0));
-    double wr = cr * sqrt(1.0 + g1 * (pst / pr - 1.0));
-    double usl = ul - (pst - pl) / wl;
-    double usr = ur + (pst - pr) / wr;
-    double zl = 2.0 * wl * wl * wl / (wl * wl + cl * cl);
-    double zr = 2.0 * wr * wr * wr / (wr * wr + cr * cr);
-    double pnew = pst - zl * zr * (usr - usl) / (zl + zr);
+    double wl = cl * soft_sqrt(1.0 + g1 * (soft_div(pst, pl) - 1.0));
+    double wr = cr * soft_sqrt(1.0 + g1 * (soft_div(pst, pr) - 1.0));
+    double usl = ul - soft_div(pst - pl, wl);
+    double usr = ur + soft_div(pst - pr, wr);
+    double zl = soft_div(2.0 * wl * wl * wl, wl * wl + cl * cl);
+    double zr = soft_div(2.0 * wr * wr * wr, wr * wr + cr * cr);
+    double pnew = pst - soft_div(zl * zr * (usr - usl), zl + zr);
     pnew = pnew < s.small_pres ? s.small_pres : pnew;
     double dp = fabs(pnew - pst);
     pst = pnew;
     ++it;
-    if (dp <= s.tol * pst || dp * (zl + zr) / (zl * zr) <= s.tol * vscale) {
+    if (dp <= s.tol * pst || soft_div(dp * (zl + zr), zl * zr) <= s.tol * vscale) {
       ok = true;
       break;
     }
   }
   iters = it;
   conv = ok;
-  const double wl = cl * sqrt(1.0 + g1 * (pst / pl - 1.0));
-  const double wr = cr * sqrt(1.0 + g1 * (pst / pr - 1.0));
-  const double ust = ((wl * ul + wr * ur) + (pl - pr)) / (wl + wr);
+  const double wl = cl * soft_sqrt(1.0 + g1 * (soft_div(pst, pl) - 1.0));
+  const double wr = cr * soft_sqrt(1.0 + g1 * (soft_div(pst, pr) - 1.0));
+  const double ust = soft_div((wl * ul + wr * ur) + (pl - pr), wl + wr);
 
   double fr, fu, fv, fp;
   if (ust == 0.0) {
@@ -762,18 +769,18 @@ __device__ __forceinline__ void riemann(const SP<double>& s, const double qL[4],
     const double sgn = left ? 1.0 : -1.0;
     const double ro = left ? rl : rr, uo = left ? ul : ur, vo = left ? vl : vr, po = left ? pl : pr;
     const double wo = left ? wl : wr;
-    const double rst = 1.0 / (1.0 / ro - (pst - po) / (wo * wo));
+    const double rst = soft_div(1.0, soft_div(1.0, ro) - soft_div(pst - po, wo * wo));
     fv = vo;
     if (pst > po) {
-      const double S = uo - sgn * (wo / ro);
+      const double S = uo - sgn * soft_div(wo, ro);
       if (sgn * S >= 0.0) {
         fr = ro; fu = uo; fp = po;
       } else {
         fr = rst; fu = ust; fp = pst;
       }
     } else {
-      const double co = sqrt(g * po / ro);
-      const double cst = sqrt(g * pst / rst);
+      const double co = soft_sqrt(soft_div(g * po, ro));
+      const double cst = soft_sqrt(soft_div(g * pst, rst));
       const double SH = uo - sgn * co;
       const double ST = ust - sgn * cst;
       if (sgn * SH >= 0.0) {
@@ -781,7 +788,7 @@ __device__ __forceinline__ void riemann(const SP<double>& s, const double qL[4],
       } else if (sgn * ST <= 0.0) {
         fr = rst; fu = ust; fp = pst;
       } else {
-        const double frac = SH / (SH - ST);
+        const double frac = soft_div(SH, SH - ST);
         fr = ro + frac * (rst - ro);
         fu = uo + frac * (ust - uo);
         fp = po + frac * (pst - po);
@@ -909,8 +916,8 @@ __device__ __forceinline__ void hllc(const SP<R>& s, const R qL[4], const R qR[4
     cl = M<R>::sq(s.gamma * pl * rcpa(rl));
     cr = M<R>::sq(s.gamma * pr * rcpa(rr));
   } else {
-    cl = sqrt(s.gamma * pl / rl);
-    cr = sqrt(s.gamma * pr / rr);
+    cl = soft_sqrt(soft_div(s.gamma * pl, rl));
+    cr = soft_sqrt(soft_div(s.gamma * pr, rr));
   }
   const R SL = M<R>::mn(ul - cl, ur - cr);
   const R SR = M<R>::mx(ul + cl, ur + cr);
@@ -920,7 +927,7 @@ __device__ __forceinline__ void hllc(const SP<R>& s, const R qL[4], const R qR[4
   if constexpr (is_f32<R>())
     sst = num * rcpa(den);
   else
-    sst = num / den;
+    sst = soft_div(num, den);
   // side whose flux the face takes (left when the whole fan is right of it, or the contact is), and whether
   // that side's outer wave has passed the face
   const bool left = (R)0 <= SL || (R)0 <= sst;
@@ -936,9 +943,9 @@ __device__ __forceinline__ void hllc(const SP<R>& s, const R qL[4], const R qR[4
       f = a * rcpa(So - sst);
       es = Eo * rcpa(ro) + (sst - uo) * (sst + po * rcpa(a));
     } else {
-      Eo = po / s.gm1 + 0.5 * ro * (uo * uo + vo * vo);
-      f = ro * (So - uo) / (So - sst);
-      es = Eo / ro + (sst - uo) * (sst + po / (ro * (So - uo)));
+      Eo = soft_div(po, s.gm1) + 0.5 * ro * (uo * uo + vo * vo);
+      f = soft_div(ro * (So - uo), So - sst);
+      es = soft_div(Eo, ro) + (sst - uo) * (sst + soft_div(po, ro * (So - uo)));
     }
     const R Us[4] = {f, f * sst, f * vo, f * es};
     const R Uo[4] = {ro, ro * uo, ro * vo, Eo};
@@ -988,12 +995,12 @@ __device__ __forceinline__ void cfl_value(const SP<R>& s, R U0, R U1, R U2, R U3
     R rho, u, v, p;
     cons_to_prim(s, U0, U1, U2, U3, rho, u, v, p);
     {
-      const R ke = (0.5 * (U1 * U1 + U2 * U2)) / U0;
+      const R ke = soft_div(0.5 * (U1 * U1 + U2 * U2), U0);
       if (!(U0 > (R)0) || !(U3 - ke > (R)0)) flags |= STATUS_NEGATIVE;
     }
-    const R cs = sqrt((s.gamma * p) / rho);
-    const R tx = s.dx / (fabs(u) + cs);
-    const R ty = s.dy / (fabs(v) + cs);
+    const R cs = soft_sqrt(soft_div(s.gamma * p, rho));
+    const R tx = soft_div(s.dx, fabs(u) + cs);
+    const R ty = soft_div(s.dy, fabs(v) + cs);
     const R t = fmin(tx, ty);
     rbest = t < rbest ? t : rbest;
   }

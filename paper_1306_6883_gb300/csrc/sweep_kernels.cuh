@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
       if constexpr (is_f32<R>()) {
         av = s.cvisc * M<R>::mx(sun[cL] - sun[cR], (R)0);
       } else {
-        const R div = (sun[cR] - sun[cL]) / h;
+        const R div = soft_div(sun[cR] - sun[cL], h);
         av = s.cvisc * M<R>::mx(-div * h, (R)0);
       }
       R UL[4], UR[4];
