@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) batch_dt_kernel(const BatchMember* __rest
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const R o = __shfl_xor_sync(0xffffffffu, rbest, off);
-    rbest = o < rbest ? o : rbest;
+    rbest = M<R>::mnp(o, rbest);
     flags |= __shfl_xor_sync(0xffffffffu, flags, off);
   }
   __shared__ R wmin[8];
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(NT, is_f32<R>() ? 3 : 2) batch_step_kernel(con
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
-      cmin = o < cmin ? o : cmin;
+      cmin = M<R>::mnp(o, cmin);
     }
     if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = cmin;
     __syncthreads();

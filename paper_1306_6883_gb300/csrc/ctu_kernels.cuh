@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R>()) ctu_step_fused_kernel(KPa
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
-    cmin = o < cmin ? o : cmin;
+    cmin = M<R>::mnp(o, cmin);
   }
   __shared__ R wmin[NT / 32];
   __shared__ bool last;

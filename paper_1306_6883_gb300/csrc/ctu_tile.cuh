@@ -352,11 +352,11 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
         return flatten_chi<R>(qp[b + (m - 2) * QP], qp[b + (m - 1) * QP], qp[b + (m + 1) * QP], qp[b + (m + 2) * QP],
                               qv[b + (m - 1) * QP], qv[b + (m + 1) * QP], s.small_pres);
       };
-      const int sx = (qp[b + 1] - qp[b - 1]) >= (R)0 ? 1 : -1;
-      const int sy = (qp[b + QP] - qp[b - QP]) >= (R)0 ? 1 : -1;
-      const R xix = M<R>::mn(chix(0), chix(-sx));
-      const R xiy = M<R>::mn(chiy(0), chiy(-sy));
-      xi = M<R>::mn(xix, xiy);
+      const int sx = M<R>::ge0(qp[b + 1] - qp[b - 1]) ? 1 : -1;
+      const int sy = M<R>::ge0(qp[b + QP] - qp[b - QP]) ? 1 : -1;
+      const R xix = M<R>::mnp(chix(0), chix(-sx));
+      const R xiy = M<R>::mnp(chiy(0), chiy(-sy));
+      xi = M<R>::mnp(xix, xiy);
     }
     sxi[e] = xi;
     su[e] = qu[b];
@@ -622,7 +622,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
             div = (su[cR] - su[cL]) * s.idx + dvy * (0.25f * s.idy);
           else
             div = soft_div(su[cR] - su[cL], s.dx) + soft_div(dvy, 4.0 * s.dy);
-          const R av = s.cvisc * M<R>::mx(-div * s.dx, (R)0);
+          const R av = s.cvisc * M<R>::mx0(-div * s.dx);
           if constexpr (L::SMEM_U) {
             R uL[4], uR[4], du[4];
             Quad<R, nC>::ld(sU, cL, uL);
@@ -651,7 +651,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
             div = (sv[cR] - sv[cL]) * s.idy + dux * (0.25f * s.idx);
           else
             div = soft_div(sv[cR] - sv[cL], s.dy) + soft_div(dux, 4.0 * s.dx);
-          const R av = s.cvisc * M<R>::mx(-div * s.dy, (R)0);
+          const R av = s.cvisc * M<R>::mx0(-div * s.dy);
           if constexpr (L::SMEM_U) {
             R uL[4], uR[4], du[4];
             Quad<R, nC>::ld(sU, cL, uL);
@@ -746,8 +746,8 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
     } else if (!finite4(Un[0], Un[1], Un[2], Un[3])) {
       flags |= STATUS_NONFINITE;
     } else {
-      const R ke = M<R>::dv((R)0.5 * (Un[1] * Un[1] + Un[2] * Un[2]), Un[0]);
-      if (!(Un[0] > (R)0) || !(Un[3] - ke > (R)0)) flags |= STATUS_NEGATIVE;
+      const R ke = M<R>::dv(M<R>::half(Un[1] * Un[1] + Un[2] * Un[2]), Un[0]);
+      if (!M<R>::gt0(Un[0]) || !M<R>::gt0(Un[3] - ke)) flags |= STATUS_NEGATIVE;
     }
   }
 }

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(DT_THREADS) cfl_dt_kernel(KParams P, const R* 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const R o = __shfl_xor_sync(0xffffffffu, rbest, off);
-    rbest = o < rbest ? o : rbest;
+    rbest = M<R>::mnp(o, rbest);
     flags |= __shfl_xor_sync(0xffffffffu, flags, off);
   }
   const double best = (double)rbest;

@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
         return flatten_chi<R>(qp[b + (m - 2) * st], qp[b + (m - 1) * st], qp[b + (m + 1) * st], qp[b + (m + 2) * st],
                               qn[b + (m - 1) * st], qn[b + (m + 1) * st], s.small_pres);
       };
-      const int sgn = (qp[b + st] - qp[b - st]) >= (R)0 ? 1 : -1;
-      xi = M<R>::mn(chi(0), chi(-sgn));
+      const int sgn = M<R>::ge0(qp[b + st] - qp[b - st]) ? 1 : -1;
+      xi = M<R>::mnp(chi(0), chi(-sgn));
     }
     sxi[e] = xi;
     sun[e] = qn[b];
@@ -257,10 +257,10 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
     if (s.cvisc > (R)0 && valid) {
       R av;
       if constexpr (is_f32<R>()) {
-        av = s.cvisc * M<R>::mx(sun[cL] - sun[cR], (R)0);
+        av = s.cvisc * M<R>::mx0(sun[cL] - sun[cR]);
       } else {
         const R div = soft_div(sun[cR] - sun[cL], h);
-        av = s.cvisc * M<R>::mx(-div * h, (R)0);
+        av = s.cvisc * M<R>::mx0(-div * h);
       }
       R UL[4], UR[4];
       load_cell(fa - 1, l0 + l, UL);
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
       if (!finite4(Un[0], Un[1], Un[2], Un[3])) {
         cnt.flags |= STATUS_NONFINITE;
       } else {
-        const R ke = M<R>::dv((R)0.5 * (Un[1] * Un[1] + Un[2] * Un[2]), Un[0]);
-        if (!(Un[0] > (R)0) || !(Un[3] - ke > (R)0)) cnt.flags |= STATUS_NEGATIVE;
+        const R ke = M<R>::dv(M<R>::half(Un[1] * Un[1] + Un[2] * Un[2]), Un[0]);
+        if (!M<R>::gt0(Un[0]) || !M<R>::gt0(Un[3] - ke)) cnt.flags |= STATUS_NEGATIVE;
       }
     }
   }
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
-      cmin = o < cmin ? o : cmin;
+      cmin = M<R>::mnp(o, cmin);
     }
     __shared__ R wmin[NT / 32];
     __shared__ bool last;
