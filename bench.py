@@ -853,7 +853,7 @@ def run_ours(args, world, rank, local):
     rl_plain = roofline("fp32", zones, sum(plain["step_ms"]) / len(plain["step_ms"]), plain["iters_per_solve"],
                         "ctu_step_fused_kernel<float, 32, 16, 384, FACE_PLAIN>")
     rl_64 = roofline("fp64", zones, sum(fp64["step_ms"]) / len(fp64["step_ms"]), fp64["iters_per_solve"],
-                     "ctu_step_fused_kernel<double, 16, 16, 256, FACE_PLAIN>")
+                     "ctu_step_fused_kernel<double, 16, 16, 384, FACE_PLAIN>")
 
     secondary = {}
     secondary["kh1024"] = kh_line(flush, 40, args.warmup)

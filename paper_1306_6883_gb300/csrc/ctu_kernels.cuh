@@ -69,15 +69,25 @@ constexpr int F32_TX = HYDRO_F32_TX, F32_TY = HYDRO_F32_TY, F32_NT = HYDRO_F32_N
 #ifndef HYDRO_F32_MINB
 #define HYDRO_F32_MINB 3
 #endif
-// Resident blocks per SM the register allocator must allow: shared memory admits three tiles per SM in
-// both precisions, and three blocks of 384 (FP32) or 256 (FP64) threads need <= 56 or <= 85 registers.
-template <typename R>
+// Tiles of the FP64 kernels.  Their time is the SM's one FP64 unit, so a tile's cost is its FP64 instructions,
+// and what counts is the halo (for large grids) or how many SMs have a tile at all (for small ones).  Measured on
+// KH 1024^2 per step / Sod 128^2 host loop per step: 16x16 at 384 threads, two per SM 2.75 ms / 155 us; at 256
+// threads, three per SM 2.95 / 204; 32x8 at 384 2.74 / 155; 32x16 at 512, one per SM 2.84 / 267; 16x8 at 384
+// 3.72 / 109; 16x8 at 192 3.32 / 119; 8x8 at 256 4.06 / 119.  A 16x8 tile costs 0.68 of a 16x16 one in both
+// columns, so a step takes the shape with the smaller (tiles per SM, rounded up) x cost: 16x8 while its tiles
+// find an SM each that 16x16 ones would leave idle.
+constexpr int F64_TX = 16, F64_TY = 16, F64_NT = 384, F64_TY_SMALL = 8;
+
+// Resident blocks per SM the register allocator must allow: shared memory admits three tiles per SM in FP32
+// (three blocks of 384 threads need <= 56 registers) and in FP64 two of 16x16 (<= 85 registers); the small FP64
+// tile runs one to an SM.
+template <typename R, int TY>
 constexpr int min_blocks() {
-  return is_f32<R>() ? HYDRO_F32_MINB : 3;
+  return is_f32<R>() ? HYDRO_F32_MINB : TY == F64_TY ? 2 : 1;
 }
 
 template <typename R, int TX, int TY, int NT, int MODE>
-__global__ void __launch_bounds__(NT, min_blocks<R>()) ctu_step_kernel(KParams P, const R* __restrict__ Uin, R* __restrict__ Uout,
+__global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_kernel(KParams P, const R* __restrict__ Uin, R* __restrict__ Uout,
                                                       StepScalars sc_host, const StepScalars* __restrict__ sc_dev,
                                                       DevScratch* __restrict__ scr, FaceHook hook,
                                                       const __grid_constant__ CUtensorMap tmap, int use_tma) {
@@ -129,7 +139,7 @@ cudaError_t launch_ctu_step(const KParams& P, const R* Uin, R* Uout, const StepS
 // split into launches over bands of tile rows (by0: the band's first tile row; nblocks: the tiles of the
 // whole step), which run concurrently; the last block of all of them finishes the step.
 template <typename R, int TX, int TY, int NT, int MODE = FACE_PLAIN>
-__global__ void __launch_bounds__(NT, min_blocks<R>()) ctu_step_fused_kernel(KParams P, const R* __restrict__ Uin,
+__global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_fused_kernel(KParams P, const R* __restrict__ Uin,
                                                             R* __restrict__ Uout, const StepScalars* __restrict__ sc_cur,
                                                             StepScalars* __restrict__ sc_next,
                                                             DevScratch* __restrict__ scr, double tmax,
@@ -146,7 +156,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R>()) ctu_step_fused_kernel(KPa
   TileCounters cnt;
   R cmin = is_f32<R>() ? (R)FLT_MAX : (R)DBL_MAX;
   const int by = by0 + (int)blockIdx.y;
-  if (sc_cur->dt == 0.0) {
+  if (sf_zero(sc_cur->dt)) {
     // a step of length zero (the run has reached tmax) leaves the state as it is: copy the tile's interior
     // cells and take their CFL constraint as a step would (the next dt is then clamped to 0 again)
     const size_t plane = (size_t)P.NY * P.pitch;
@@ -218,6 +228,44 @@ cudaError_t launch_ctu_step_fused(const KParams& P, const R* Uin, R* Uout, const
       P, Uin, Uout, sc_cur, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
       (unsigned int)tx * (unsigned int)ty, mlp);
   return cudaGetLastError();
+}
+
+// Whether an FP64 step takes 16x8 tiles instead of 16x16 ones (see F64_TY_SMALL).
+inline cudaError_t f64_small_tile(const KParams& P, bool* small) {
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  auto rounds = [&](int ty) {
+    const long long n = (long long)((P.nx + F64_TX - 1) / F64_TX) * ((P.ny + ty - 1) / ty);
+    return (n + nsm - 1) / nsm;
+  };
+  *small = 17 * rounds(F64_TY_SMALL) < 25 * rounds(F64_TY);
+  return cudaSuccess;
+}
+
+template <int MODE>
+cudaError_t launch_ctu_step_f64(const KParams& P, const double* Uin, double* Uout, const StepScalars& sc_host,
+                                const StepScalars* sc_dev, DevScratch* scr, cudaStream_t stream) {
+  bool small = false;
+  const cudaError_t e = f64_small_tile(P, &small);
+  if (e != cudaSuccess) return e;
+  const auto launch = small ? launch_ctu_step<double, F64_TX, F64_TY_SMALL, F64_NT, MODE>
+                            : launch_ctu_step<double, F64_TX, F64_TY, F64_NT, MODE>;
+  return launch(P, Uin, Uout, sc_host, sc_dev, scr, FaceHook{}, nullptr, stream);
+}
+
+// A band of a step (band.y > 0) counts tile rows of 16 cells (fused_tile_height).
+template <int MODE>
+cudaError_t launch_ctu_step_fused_f64(const KParams& P, const double* Uin, double* Uout, const StepScalars* sc_cur,
+                                      StepScalars* sc_next, DevScratch* scr, double tmax, cudaStream_t stream,
+                                      int2 band) {
+  bool small = false;
+  const cudaError_t e = band.y > 0 ? cudaSuccess : f64_small_tile(P, &small);
+  if (e != cudaSuccess) return e;
+  const auto launch = small ? launch_ctu_step_fused<double, F64_TX, F64_TY_SMALL, F64_NT, MODE>
+                            : launch_ctu_step_fused<double, F64_TX, F64_TY, F64_NT, MODE>;
+  return launch(P, Uin, Uout, sc_cur, sc_next, scr, tmax, nullptr, stream, band, nullptr);
 }
 
 }  // namespace hydro

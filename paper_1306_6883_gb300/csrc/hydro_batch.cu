@@ -337,7 +337,7 @@ hydro_status hydro_batch_class_info(const hydro_batch* b, int k, int* nx, int* n
                                     int* tile_y, int* threads) {
   if (!b || k < 0 || k >= (int)b->classes.size()) return HYDRO_EINVAL;
   const SizeClass& c = b->classes[k];
-  const hydro::TileShape ts = b->precision == HYDRO_FP64 ? hydro::TileShape{16, 16, 256} : hydro::kTileShapes[c.shape];
+  const hydro::TileShape ts = b->precision == HYDRO_FP64 ? hydro::TileShape{16, 16, 384} : hydro::kTileShapes[c.shape];
   if (nx) *nx = c.nx;
   if (ny) *ny = c.ny;
   if (members) *members = (int)c.members.size();

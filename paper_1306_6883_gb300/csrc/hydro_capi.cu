@@ -871,7 +871,7 @@ hydro_status hydro_step_host_chained(hydro_ctx* c, const void* host_in, void* ho
 const char* hydro_last_error(const hydro_ctx* c) { return c ? c->err : "no context"; }
 
 const char* hydro_build_info(void) {
-  return "hydro sm_103a; kernels: fill_ghost, cfl_dt, ctu_step and ctu_step_fused (fp64 16x16/256 exact rounding, "
+  return "hydro sm_103a; kernels: fill_ghost, cfl_dt, ctu_step and ctu_step_fused (fp64 16x16/384 or 16x8/384 exact rounding, "
          "fp32 32x16/384 with TMA tile loads), batch fill/dt/step, totals, mlp";
 }
 

@@ -26,7 +26,7 @@ cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, voi
                                                               tmax, tmap, stream, band);
 }
 
-int fused_tile_height(int precision) { return precision == 0 ? 16 : F32_TY; }  // FP64 tiles are 16 x 16
+int fused_tile_height(int precision) { return precision == 0 ? F64_TY : F32_TY; }
 
 int fused_tile_rows(int precision, const KParams& P) {
   const int th = fused_tile_height(precision);
