@@ -13,8 +13,7 @@ namespace hydro {
 
 // Per-block reduction of the tile counters into the context's scratch: warp shuffles, then one thread adds
 // the block's sums (one atomic per counter and block; per-warp atomics on the same words cost ~4 % of a
-// KH 1024^2 step).  Called by every thread of the block.
-template <int NT>
+// KH 1024^2 step).  Called by every thread of the block (at most 512 threads).
 __device__ __forceinline__ void flush_counters(TileCounters& cnt, DevScratch* scr) {
   if (cnt.nonconv) cnt.flags |= STATUS_NONCONV;
 #pragma unroll
@@ -24,7 +23,7 @@ __device__ __forceinline__ void flush_counters(TileCounters& cnt, DevScratch* sc
     cnt.nonconv += __shfl_xor_sync(0xffffffffu, cnt.nonconv, off);
     cnt.flags |= __shfl_xor_sync(0xffffffffu, cnt.flags, off);
   }
-  __shared__ unsigned int part[NT / 32][4];
+  __shared__ unsigned int part[16][4];
   if ((threadIdx.x & 31) == 0) {
     const int w = threadIdx.x >> 5;
     part[w][0] = cnt.solves;
@@ -36,7 +35,7 @@ __device__ __forceinline__ void flush_counters(TileCounters& cnt, DevScratch* sc
   if (threadIdx.x == 0) {
     unsigned long long solves = 0, iters = 0, nonconv = 0;
     unsigned int flags = 0;
-    for (int w = 0; w < NT / 32; ++w) {
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
       solves += part[w][0];
       iters += part[w][1];
       nonconv += part[w][2];
@@ -46,6 +45,49 @@ __device__ __forceinline__ void flush_counters(TileCounters& cnt, DevScratch* sc
     atomicAdd(&scr->stats[1], iters);
     if (nonconv) atomicAdd(&scr->stats[2], nonconv);
     if (flags) atomicOr(&scr->status, flags);
+  }
+}
+
+// End of a fused step for one block: its CFL minimum into the step's accumulator and its share into the step's
+// count; the block that completes the count (total) advances the time by this step's dt and writes the next step's
+// factors.
+template <typename R>
+__device__ __forceinline__ void finish_fused_step(const KParams& P, R cmin, const StepScalars* sc_cur,
+                                                  StepScalars* sc_next, DevScratch* scr, double tmax,
+                                                  unsigned int share, unsigned int total) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
+    cmin = M<R>::mnp(o, cmin);
+  }
+  __shared__ R wmin[16];
+  __shared__ bool last;
+  if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = cmin;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    R b = wmin[0];
+    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) b = wmin[k] < b ? wmin[k] : b;
+    atomicMin(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong((double)b));
+    __threadfence();
+    last = atomicAdd(&scr->step_blocks_done, share) + share == total;
+  }
+  __syncthreads();
+  if (last && threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long bits =
+        atomicExch(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong(DBL_MAX));
+    const double t = scr->t + sc_cur->dt;
+    scr->t = t;
+    scr->nsteps = scr->nsteps + 1;
+    double dt = P.cfl * __longlong_as_double((long long)bits);
+    if (tmax > 0.0) {
+      const double left = tmax - t;
+      dt = dt > left ? left : dt;
+      dt = dt < 0.0 ? 0.0 : dt;
+    }
+    scr->dt = dt;
+    *sc_next = make_step_scalars(dt, P.dx, P.dy, P.grav);
+    scr->step_blocks_done = 0u;
   }
 }
 
@@ -102,7 +144,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_kernel(KPara
   TileCounters cnt;
   ctu_tile<R, TX, TY, NT, MODE>(P, s, f, Uin, Uout, blockIdx.x, blockIdx.y, smem_raw, cnt, hook, wsm, nullptr,
                                 use_tma ? &tmap : nullptr);
-  flush_counters<NT>(cnt, scr);
+  flush_counters(cnt, scr);
 }
 
 // Raises a kernel's dynamic shared-memory limit once per device (function attributes belong to the device's
@@ -173,41 +215,8 @@ __global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_fused_kernel
     ctu_tile<R, TX, TY, NT, MODE, true>(P, s, f, Uin, Uout, blockIdx.x, by, smem_raw, cnt, FaceHook{}, wsm,
                                         &cmin, use_tma ? &tmap : nullptr);
   }
-  flush_counters<NT>(cnt, scr);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
-    cmin = M<R>::mnp(o, cmin);
-  }
-  __shared__ R wmin[NT / 32];
-  __shared__ bool last;
-  if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = cmin;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    R b = wmin[0];
-    for (int k = 1; k < NT / 32; ++k) b = wmin[k] < b ? wmin[k] : b;
-    atomicMin(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong((double)b));
-    __threadfence();
-    last = atomicAdd(&scr->step_blocks_done, 1u) == nblocks - 1u;
-  }
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
-    __threadfence();
-    const unsigned long long bits =
-        atomicExch(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong(DBL_MAX));
-    const double t = scr->t + sc_cur->dt;
-    scr->t = t;
-    scr->nsteps = scr->nsteps + 1;
-    double dt = P.cfl * __longlong_as_double((long long)bits);
-    if (tmax > 0.0) {
-      const double left = tmax - t;
-      dt = dt > left ? left : dt;
-      dt = dt < 0.0 ? 0.0 : dt;
-    }
-    scr->dt = dt;
-    *sc_next = make_step_scalars(dt, P.dx, P.dy, P.grav);
-    scr->step_blocks_done = 0u;
-  }
+  flush_counters(cnt, scr);
+  finish_fused_step(P, cmin, sc_cur, sc_next, scr, tmax, 1u, nblocks);
 }
 
 // band: tile rows [band.x, band.x + band.y) of the step (band.y <= 0: all of them).  mlp: the network of

@@ -385,7 +385,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
           q[m] = a[0];
           ppm_edges<R>(a[-2 * st], a[-st], a[0], a[st], a[2 * st], xi, eL[m], eR[m]);
         }
-        trace_ppm<R>(s, YD ? sigy : sigx, q, eL, eR, ql, qrr);
+        trace_ppm<R>(s, YD ? sigy : sigx, q, eL, eR, Waves<R>(s, q[0], q[3]), ql, qrr);
       } else {
         R dq[4];
         if constexpr (is_f32<R>()) {
@@ -410,7 +410,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
             dq[m] = xi * slope<R>(s.limiter, a[-2 * st], a[-st], a[0], a[st], a[2 * st]);
           }
         }
-        trace<R>(s, YD ? sigy : sigx, q, dq, ql, qrr);
+        trace<R>(s, YD ? sigy : sigx, q, dq, Waves<R>(s, q[0], q[3]), ql, qrr);
       }
       if (P.use_grav) {  // half-step gravity (the rho g source, §3.2) on v: normal in y, transverse in x
         constexpr int mg = YD ? 1 : 2;

@@ -293,6 +293,15 @@ __device__ __forceinline__ void fill_ghost_cell(const KParams& P, R* __restrict_
 }
 
 // ---------------------------------------------------------------------------------------------------
+// Pressure (gamma - 1)(E - |m|^2 / (2 rho)) in double from float values.  Every product, sum and quotient rounds on
+// its own, so that all callers get the same value.  Not inlined: its two divisions are some 300 instructions, which
+// every inlined copy would put between the common path's (cons_to_prim 336 -> 64 instructions).
+static __device__ __noinline__ float recovered_pressure_f64(float gm1, float rho, float mx, float my, float E) {
+  const double rd = (double)rho, ud = __ddiv_rn((double)mx, rd), vd = __ddiv_rn((double)my, rd);
+  const double ke = __dmul_rn(__dmul_rn(0.5, rd), __dadd_rn(__dmul_rn(ud, ud), __dmul_rn(vd, vd)));
+  return (float)__dmul_rn((double)gm1, __dsub_rn((double)E, ke));
+}
+
 // EOS (Eqs. 11-12): conserved (rho, mx, my, E) -> primitive (rho, u, v, p), floors on the copy.
 template <typename R>
 __device__ __forceinline__ void cons_to_prim(const SP<R>& s, R U0, R U1, R U2, R U3, R& rho, R& u, R& v, R& p) {
@@ -302,15 +311,10 @@ __device__ __forceinline__ void cons_to_prim(const SP<R>& s, R U0, R U1, R U2, R
     const float2 uv = mul2(f2(U1, U2), f2(ir));
     u = uv.x;
     v = uv.y;
-    const float ke = 0.5f * rho * (u * u + v * v);
-    if (ke > s.rec * U3) {
-      // kinetic energy within 0.1% (by default) of the total: recover e = E - rho |u|^2 / 2 in double
-      const double rd = (double)rho, ud = (double)U1 / rd, vd = (double)U2 / rd;
-      const double ked = 0.5 * rd * (ud * ud + vd * vd);
-      p = (float)(((double)s.gm1) * ((double)U3 - ked));
-    } else {
-      p = s.gm1 * (U3 - ke);
-    }
+    const float ke = __fmul_rn(0.5f * rho, __fmaf_rn(u, u, __fmul_rn(v, v)));  // the same in every instance
+    p = __fmul_rn(s.gm1, __fsub_rn(U3, ke));
+    // kinetic energy within 0.1% (by default) of the total: recover e = E - rho |u|^2 / 2 in double
+    if (ke > s.rec * U3) p = recovered_pressure_f64(s.gm1, rho, U1, U2, U3);
   } else {
     u = soft_div(U1, rho);
     v = soft_div(U2, rho);
@@ -355,22 +359,29 @@ static __device__ __noinline__ float corrected_pressure_f64(float gm1, float igm
 // round trip through E does not cancel the pressure away (high Mach).
 template <typename R>
 __device__ __forceinline__ void correct_state(const SP<R>& s, R rho, R u, R v, R p, const R dF[4], R h, R q[4]) {
-  R U[4];
   if constexpr (is_f32<R>()) {
-    // prim_to_cons, keeping the kinetic energy for the high-Mach test
+    // prim_to_cons, the correction and cons_to_prim, with one test for both high-Mach cases
     const float ke = 0.5f * rho * (u * u + v * v);
-    U[0] = rho;
-    U[1] = rho * u;
-    U[2] = rho * v;
-    U[3] = p * s.igm1 + ke;
-    const bool high_mach = ke > s.rec * U[3];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) U[k] = U[k] - h * dF[k];
-    cons_to_prim(s, U[0], U[1], U[2], U[3], q[0], q[1], q[2], q[3]);
-    if (high_mach)
-      q[3] = corrected_pressure_f64(s.gm1, s.igm1, s.small_dens, s.small_pres, rho, u, v, p, h, dF[0], dF[1], dF[2],
-                                    dF[3]);
+    const float2 m = mul2(f2(rho), f2(u, v));
+    const float E0 = p * s.igm1 + ke;
+    const float r = rho - h * dF[0];
+    const float2 m2 = fma2(f2(-h), f2(dF[1], dF[2]), m);
+    const float E = E0 - h * dF[3];
+    const float rf = r < s.small_dens ? s.small_dens : r;
+    const float2 w = mul2(m2, f2(rcpa(rf)));
+    const float ke2 = 0.5f * rf * (w.x * w.x + w.y * w.y);
+    float pc = s.gm1 * (E - ke2);
+    const bool before = ke > s.rec * E0, after = ke2 > s.rec * E;
+    if (before || after)
+      pc = before ? corrected_pressure_f64(s.gm1, s.igm1, s.small_dens, s.small_pres, rho, u, v, p, h, dF[0], dF[1],
+                                           dF[2], dF[3])
+                  : recovered_pressure_f64(s.gm1, rf, m2.x, m2.y, E);
+    q[0] = rf;
+    q[1] = w.x;
+    q[2] = w.y;
+    q[3] = pc < s.small_pres ? s.small_pres : pc;
   } else {
+    R U[4];
     prim_to_cons(s, rho, u, v, p, U[0], U[1], U[2], U[3]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) U[k] = U[k] - h * dF[k];
@@ -427,7 +438,7 @@ __device__ __forceinline__ float2 mc2_pair(float2 qm, float2 q0, float2 qp) {
   const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl.x), fabsf(dr.x)), fminf(fabsf(dl.y), fabsf(dr.y))));
   const float2 pr = mul2(dl, dr);
   const float mx = fminf(fabsf(dc.x), dlim.x), my = fminf(fabsf(dc.y), dlim.y);
-  return f2(pr.x > 0.f ? (dc.x >= 0.f ? mx : -mx) : 0.f, pr.y > 0.f ? (dc.y >= 0.f ? my : -my) : 0.f);
+  return f2(pr.x > 0.f ? copysignf(mx, dc.x) : 0.f, pr.y > 0.f ? copysignf(my, dc.y) : 0.f);
 }
 
 __device__ __forceinline__ float2 slope_pair(int limiter, float2 qm2, float2 qm1, float2 q0, float2 qp1, float2 qp2) {
@@ -439,7 +450,58 @@ __device__ __forceinline__ float2 slope_pair(int limiter, float2 qm2, float2 qm1
   const float2 d4 = fma2(f2(4.0f / 3.0f), dc, mul2(f2(-1.0f / 6.0f), m));
   const float2 pr = mul2(dl, dr);
   const float mx = fminf(fabsf(d4.x), dlim.x), my = fminf(fabsf(d4.y), dlim.y);
-  return f2(pr.x > 0.f ? (d4.x >= 0.f ? mx : -mx) : 0.f, pr.y > 0.f ? (d4.y >= 0.f ? my : -my) : 0.f);
+  return f2(pr.x > 0.f ? copysignf(mx, d4.x) : 0.f, pr.y > 0.f ? copysignf(my, d4.y) : 0.f);
+}
+
+// The limiter of four components at once from their one-sided differences dl = q0 - qm, dr = qp - q0 and
+// dd = qp - qm: the MC slopes (mc4), and the fourth-order slopes times xi from them and the neighbours' MC slopes
+// (slope4), with the operations and order of mc2, slope and slope_pair.
+template <typename R>
+__device__ __forceinline__ void mc4(const R dl[4], const R dr[4], const R dd[4], R m[4]) {
+  if constexpr (is_f32<R>()) {
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+      const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
+      const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
+      const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
+      const float mx = fminf(fabsf(dc.x), dlim.x), my = fminf(fabsf(dc.y), dlim.y);
+      m[h] = pr.x > 0.f ? copysignf(mx, dc.x) : 0.f;
+      m[h + 1] = pr.y > 0.f ? copysignf(my, dc.y) : 0.f;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = limited64(dl[k], dr[k], sf_half(dd[k]));
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void slope4(int limiter, R xi, const R dl[4], const R dr[4], const R dd[4], const R mL[4],
+                                       const R m0[4], const R mR[4], R dq[4]) {
+  if (limiter != 2) {  // uniform over the launch: piecewise constant (0) or MC (1)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dq[k] = limiter == 0 ? (R)0 : xi * m0[k];
+    return;
+  }
+  if constexpr (is_f32<R>()) {
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+      const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
+      const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
+      const float2 m = add2(f2(mR[h], mR[h + 1]), f2(mL[h], mL[h + 1]));
+      const float2 d4 = fma2(f2(4.0f / 3.0f), dc, mul2(f2(-1.0f / 6.0f), m));
+      const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
+      const float mx = fminf(fabsf(d4.x), dlim.x), my = fminf(fabsf(d4.y), dlim.y);
+      const float2 d = mul2(f2(xi), f2(pr.x > 0.f ? copysignf(mx, d4.x) : 0.f, pr.y > 0.f ? copysignf(my, d4.y) : 0.f));
+      dq[h] = d.x;
+      dq[h + 1] = d.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double d4 = (4.0 / 3.0) * sf_half(dd[k]) - (1.0 / 6.0) * (mR[k] + mL[k]);
+      dq[k] = xi * limited64(dl[k], dr[k], d4);
+    }
+  }
 }
 
 // Flattening shock detector on one line (§3.2, Colella 1990): chi in [0, 1].
@@ -460,7 +522,7 @@ __device__ __forceinline__ R flatten_chi(R pm2, R pm1, R pp1, R pp2, R um1, R up
   R chi;
   if constexpr (is_f32<R>()) {
     const float z = M<float>::ab(dp1) * rcpa(M<float>::mx(M<float>::ab(dp2), small_pres));
-    chi = 1.0f - (z - z0) * (1.0f / (0.85f - 0.75f));
+    chi = __fmaf_rn(-__fsub_rn(z, z0), 1.0f / (0.85f - 0.75f), 1.0f);
   } else {
     R z = soft_div(M<R>::ab(dp1), M<R>::mx(M<R>::ab(dp2), small_pres));
     chi = (R)1 - soft_div(z - z0, z1 - z0);
@@ -478,28 +540,38 @@ __device__ __forceinline__ R flatten_chi(R pm2, R pm1, R pp1, R pp2, R um1, R up
 // Left state at i+1/2: q + (1 - sigma lam4) dq/2 + sum over lam_nu >= 0 of (sigma/2)(lam4 - lam_nu) beta_nu r_nu.
 // Right state at i-1/2: q - (1 + sigma lam1) dq/2 + sum over lam_nu <= 0 of (sigma/2)(lam1 - lam_nu) beta_nu r_nu.
 // Only the non-zero eigenvector entries are multiplied out.
+// The direction-independent part of the tracing: sound speed c and the non-zero eigenvector factors
+// c^2, rho/2c, 1/2c^2, 1/c^2, c/rho of a cell (rho, p).
 template <typename R>
-__device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], const R dq[4], R qL[4], R qR[4]) {
-  const R rho = q[0], un = q[1], pres = q[3];
+struct Waves {
   R c, c2, roc, ic2h, ic2, cor;
-  if constexpr (is_f32<R>()) {
-    const float ir = rcpa(rho);
-    const float x = s.gamma * pres * ir;  // c^2
-    const float ic = rsqa(x);           // 1/c
-    c = x * ic;
-    c2 = c * c;
-    roc = 0.5f * rho * ic;
-    ic2 = ic * ic;
-    ic2h = 0.5f * ic2;
-    cor = c * ir;
-  } else {
-    c = soft_sqrt(soft_div(s.gamma * pres, rho));
-    c2 = c * c;
-    roc = soft_div(sf_half(rho), c);
-    ic2h = soft_div(0.5, c2);
-    ic2 = soft_div(1.0, c2);
-    cor = soft_div(c, rho);
+  __device__ __forceinline__ Waves(const SP<R>& s, R rho, R pres) {
+    if constexpr (is_f32<R>()) {
+      const float ir = rcpa(rho);
+      const float x = s.gamma * pres * ir;  // c^2
+      const float ic = rsqa(x);             // 1/c
+      c = x * ic;
+      c2 = c * c;
+      roc = 0.5f * rho * ic;
+      ic2 = ic * ic;
+      ic2h = 0.5f * ic2;
+      cor = c * ir;
+    } else {
+      c = soft_sqrt(soft_div(s.gamma * pres, rho));
+      c2 = c * c;
+      roc = soft_div(sf_half(rho), c);
+      ic2h = soft_div(0.5, c2);
+      ic2 = soft_div(1.0, c2);
+      cor = soft_div(c, rho);
+    }
   }
+};
+
+template <typename R>
+__device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], const R dq[4], const Waves<R>& w_, R qL[4],
+                                      R qR[4]) {
+  const R un = q[1];
+  const R c = w_.c, c2 = w_.c2, roc = w_.roc, ic2h = w_.ic2h, ic2 = w_.ic2, cor = w_.cor;
   const R lam1 = un - c, lam2 = un, lam4 = un + c;
   const R b1 = -roc * dq[1] + ic2h * dq[3];
   const R b2 = dq[0] + (-ic2) * dq[3];
@@ -526,7 +598,9 @@ __device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], con
   } else {
     l0 = q[0] + aL * dq[0]; l1 = q[1] + aL * dq[1]; l2 = q[2] + aL * dq[2]; l3 = q[3] + aL * dq[3];
   }
-  if (M<R>::ge0(lam1)) {
+  // no acoustic wave moves against the flow unless it is supersonic; FP32 skips both tests then
+  const bool supersonic = is_f32<R>() ? M<R>::ab(un) >= c : true;
+  if (supersonic && M<R>::ge0(lam1)) {
     R w = hs * g41 * b1;
     l0 += w;
     l1 += w * (-cor);
@@ -562,7 +636,7 @@ __device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], con
     R w3 = hs * g12 * b3;
     r2 += w3;
   }
-  if (M<R>::le0(lam4)) {
+  if (supersonic && M<R>::le0(lam4)) {
     R w = hs * g14 * b4;
     r0 += w;
     r1 += w * cor;
@@ -582,9 +656,9 @@ __device__ __forceinline__ void trace(const SP<R>& s, R sigma, const R q[4], con
 // a_{i+1/2} = a_i + (a_{i+1} - a_i)/2 - (da_{i+1} - da_i)/6 from MC-limited slopes da; a local extremum
 // flattens the profile to the average; a parabola whose extremum falls inside the cell has it moved to the
 // nearer edge (aL = 3 a_i - 2 aR or aR = 3 a_i - 2 aL); flattening blends the edges toward the average.
+// ppm_edges_mc: from the cell's neighbours and the three cells' MC slopes.
 template <typename R>
-__device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R& eL, R& eR) {
-  const R dm = mc2(a0, a1, a2), d0 = mc2(a1, a2, a3), dp = mc2(a2, a3, a4);
+__device__ __forceinline__ void ppm_edges_mc(R a1, R a2, R a3, R dm, R d0, R dp, R xi, R& eL, R& eR) {
   const R c = a2;
   R l, r;
   if constexpr (is_f32<R>()) {
@@ -602,16 +676,16 @@ __device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R&
   else
     d6 = soft_div(da * da, 6.0);
   const bool left_ex = da * mid > d6;
-  R d6r;
-  if constexpr (is_f32<R>())
-    d6r = -(da * da) / (R)6;
-  else
-    d6r = soft_div(-(da * da), 6.0);
-  const bool right_ex = !left_ex && d6r > da * mid;
+  const bool right_ex = !left_ex && -d6 > da * mid;
   const R l2 = flat ? c : (left_ex ? (R)3 * c - (R)2 * r : l);
   const R r2 = flat ? c : (right_ex ? (R)3 * c - (R)2 * l : r);
   eL = xi * l2 + ((R)1 - xi) * c;
   eR = xi * r2 + ((R)1 - xi) * c;
+}
+
+template <typename R>
+__device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R& eL, R& eR) {
+  ppm_edges_mc<R>(a1, a2, a3, mc2(a0, a1, a2), mc2(a1, a2, a3), mc2(a2, a3, a4), xi, eL, eR);
 }
 
 // PPM characteristic tracing in the face frame.  The cell's profile is a(x) = aL + x (da + a6 (1 - x)) on
@@ -623,27 +697,9 @@ __device__ __forceinline__ void ppm_edges(R a0, R a1, R a2, R a3, R a4, R xi, R&
 // order of the wave sums); floors on the results.
 template <typename R>
 __device__ __forceinline__ void trace_ppm(const SP<R>& s, R sigma, const R q[4], const R eL[4], const R eR[4],
-                                          R qL[4], R qR[4]) {
-  const R rho = q[0], un = q[1], pres = q[3];
-  R c, c2, roc, ic2h, ic2, cor;
-  if constexpr (is_f32<R>()) {
-    const float ir = rcpa(rho);
-    const float x = s.gamma * pres * ir;
-    const float ic = rsqa(x);
-    c = x * ic;
-    c2 = c * c;
-    roc = 0.5f * rho * ic;
-    ic2 = ic * ic;
-    ic2h = 0.5f * ic2;
-    cor = c * ir;
-  } else {
-    c = soft_sqrt(soft_div(s.gamma * pres, rho));
-    c2 = c * c;
-    roc = soft_div(sf_half(rho), c);
-    ic2h = soft_div(0.5, c2);
-    ic2 = soft_div(1.0, c2);
-    cor = soft_div(c, rho);
-  }
+                                          const Waves<R>& w_, R qL[4], R qR[4]) {
+  const R un = q[1];
+  const R c = w_.c, c2 = w_.c2, roc = w_.roc, ic2h = w_.ic2h, ic2 = w_.ic2, cor = w_.cor;
   const R lam1 = un - c, lam2 = un, lam4 = un + c;
   R da[4], a6[4];
 #pragma unroll
@@ -848,99 +904,147 @@ static __device__ __noinline__ void riemann(const SP<double>& s, const double qL
 // FP32 form of the same solver.  With a_K = 1 + (gamma+1)/(2 gamma)(p/p_K - 1) and t_K = 1/sqrt(a_K):
 // 1/W_K = t_K / C_K, W_K = C_K a_K t_K, and the Newton step -(u*_R - u*_L) / (1/Z_L + 1/Z_R) uses
 // 1/Z_K = (a_K + 1) t_K^3 / (2 C_K); one rsqrt per side and one reciprocal per iteration.
-__device__ __forceinline__ void riemann(const SP<float>& s, const float qL[4], const float qR[4], float guess,
-                                        float F[4], int& iters, bool& conv, float* pstar_out = nullptr) {
-  const float g = s.gamma, g1 = s.g1;
-  const float rl = qL[0], ul = qL[1], vl = qL[2], pl = qL[3];
-  const float rr = qR[0], ur = qR[1], vr = qR[2], pr = qR[3];
-  // the two sides go through the same arithmetic: (left, right) pairs in packed operations
-  const float2 P = f2(pl, pr), U = f2(ul, ur);
-  const float2 X = mul2(mul2(f2(g), P), f2(rl, rr));  // C_K^2 = gamma p_K rho_K
-  const float icl = rsqa(X.x), icr = rsqa(X.y);       // 1/C_K
-  const float2 C = mul2(X, f2(icl, icr));
-  const float cl = C.x, cr = C.y;
-  // one MUFU reciprocal each costs fewer issue slots than forming 1/p_K from 1/C_K^2 = 1/(gamma p_K rho_K)
-  const float2 IP = f2(rcpa(pl), rcpa(pr));
-  // velocity scale of the problem: float rounding leaves u*_R - u*_L uncertain by ~2^-24 of it, which can
-  // exceed tol * p* in pressure when p* << rho u^2, so the FP32 stopping rule also accepts a pressure
-  // change smaller than the one a velocity mismatch of tol times this scale would produce
-  const float2 PIC = mul2(P, f2(icl, icr));
-  const float tolv = s.tol * (fabsf(ul) + fabsf(ur) + g * (PIC.x + PIC.y));
-  // 1/C_K with the side's sign: u*_L falls and u*_R rises with the star pressure
-  const float2 ICS = f2(-icl, icr);
-  float pst = guess > 0.0f ? guess : (cr * pl + cl * pr + cl * cr * (ul - ur)) * rcpa(cl + cr);
-  pst = pst < s.small_pres ? s.small_pres : pst;
-  int it = 0;
-  bool ok = false;
-  while (it < s.maxiter) {
-    const float2 A = fma2(f2(g1), fma2(f2(pst), IP, f2(-1.0f)), f2(1.0f));  // a_K
-    const float2 T = f2(rsqa(A.x), rsqa(A.y));                             // t_K
-    const float2 IWS = mul2(T, ICS);                                        // (-1/W_L, 1/W_R)
-    const float2 US = fma2(sub2(f2(pst), P), IWS, U);                       // (u*_L, u*_R)
+// One face of that iteration: the sides' constants, the current star pressure and the last step's size.
+struct TwoShockF {
+  float2 P, U, IC, C, IP;  // p_K, u_K, 1/C_K, C_K, 1/p_K as (left, right) pairs
+  float pst, dp, iz;
+
+  // constants of the sides and the starting pressure (acoustic unless guess > 0)
+  __device__ __forceinline__ void start(const SP<float>& s, const float a[4], const float b[4], float guess) {
+    // the two sides go through the same arithmetic: (left, right) pairs in packed operations
+    P = f2(a[3], b[3]);
+    U = f2(a[1], b[1]);
+    const float2 X = mul2(mul2(f2(s.gamma), P), f2(a[0], b[0]));  // C_K^2 = gamma p_K rho_K
+    IC = f2(rsqa(X.x), rsqa(X.y));
+    C = mul2(X, IC);
+    // one MUFU reciprocal each costs fewer issue slots than forming 1/p_K from 1/C_K^2 = 1/(gamma p_K rho_K)
+    IP = f2(rcpa(P.x), rcpa(P.y));
+    pst = guess > 0.0f ? guess : (C.y * P.x + C.x * P.y + C.x * C.y * (U.x - U.y)) * rcpa(C.x + C.y);
+    pst = pst < s.small_pres ? s.small_pres : pst;
+  }
+  __device__ __forceinline__ float2 a_k(const SP<float>& s) const {
+    return fma2(f2(s.g1), fma2(f2(pst), IP, f2(-1.0f)), f2(1.0f));
+  }
+  // one Newton step
+  __device__ __forceinline__ void step(const SP<float>& s) {
+    const float2 A = a_k(s);
+    const float2 T = f2(rsqa(A.x), rsqa(A.y));            // t_K
+    const float2 IWS = mul2(T, f2(-IC.x, IC.y));          // (-1/W_L, 1/W_R): u*_L falls and u*_R rises with p*
+    const float2 US = fma2(sub2(f2(pst), P), IWS, U);     // (u*_L, u*_R)
     // (a_K + 1) t_K^2 / 2 = (1 + 1/a_K) / 2 = (1 + t_K^2) / 2
-    const float2 IZS = mul2(fma2(f2(0.5f), mul2(T, T), f2(0.5f)), IWS);    // (-1/Z_L, 1/Z_R)
-    const float iz = IZS.y - IZS.x;  // 1 / (Z_L Z_R / (Z_L + Z_R))
+    const float2 IZS = mul2(fma2(f2(0.5f), mul2(T, T), f2(0.5f)), IWS);  // (-1/Z_L, 1/Z_R)
+    iz = IZS.y - IZS.x;                                   // 1 / (Z_L Z_R / (Z_L + Z_R))
     float pnew = pst - (US.y - US.x) * rcpa(iz);
     pnew = pnew < s.small_pres ? s.small_pres : pnew;
-    const float dp = fabsf(pnew - pst);
+    dp = fabsf(pnew - pst);
     pst = pnew;
-    ++it;
-    if (dp <= s.tol * pst || dp * iz <= tolv) {
-      ok = true;
-      break;
-    }
   }
-  iters = it;
-  conv = ok;
-  const float2 A = fma2(f2(g1), fma2(f2(pst), IP, f2(-1.0f)), f2(1.0f));
-  const float tl = rsqa(A.x), tr = rsqa(A.y);
-  const float2 W = mul2(mul2(C, A), f2(tl, tr));
-  const float wl = W.x, wr = W.y;
-  const float2 WU = mul2(W, U);
-  const float ust = ((WU.x + WU.y) + (pl - pr)) * rcpa(wl + wr);
-
-  // sampling at x/t = 0 (the same cases as the FP64 solver).  A face on the contact (u* = 0; whole warps of
-  // it in a fluid at rest) takes the mean state; otherwise the case (shock, fan head, fan tail, inside the
-  // fan) is chosen by selects, since it varies within a warp and a branch per case would run every path.
-  float fr, fu, fv, fp;
-  if (ust == 0.0f) {
-    fr = 0.5f * (rl + rr);
-    fu = 0.0f;
-    fv = 0.5f * (vl + vr);
-    fp = pst;
-  } else {
+  __device__ __forceinline__ bool small_step(const SP<float>& s) const { return dp <= s.tol * pst; }
+  // velocity scale of the problem: float rounding leaves u*_R - u*_L uncertain by ~2^-24 of it, which can exceed
+  // tol * p* in pressure when p* << rho u^2, so the FP32 stopping rule also accepts a pressure change smaller
+  // than the one a velocity mismatch of tol times this scale would produce
+  __device__ __forceinline__ bool small_mismatch(const SP<float>& s) const {
+    const float2 PIC = mul2(P, IC);
+    return dp * iz <= s.tol * (fabsf(U.x) + fabsf(U.y) + s.gamma * (PIC.x + PIC.y));
+  }
+  // the rest of the iteration after a step that small_step did not end; returns the total number of steps, `it`
+  // before
+  __device__ __forceinline__ int finish(const SP<float>& s, int it, bool& ok) {
+    ok = small_mismatch(s);
+    while (!ok && it < s.maxiter) {
+      step(s);
+      ++it;
+      ok = small_step(s) || small_mismatch(s);
+    }
+    return it;
+  }
+  // star velocity; W and 1/W of both sides
+  __device__ __forceinline__ float ustar(const SP<float>& s, float2& W, float2& IW) const {
+    const float2 A = a_k(s);
+    const float2 T = f2(rsqa(A.x), rsqa(A.y));
+    W = mul2(mul2(C, A), T);
+    IW = mul2(T, IC);
+    const float2 WU = mul2(W, U);
+    return ((WU.x + WU.y) + (P.x - P.y)) * rcpa(W.x + W.y);
+  }
+  // Sampling at x/t = 0 (the same cases as the FP64 solver) of a face with u* != 0, and its flux.  The case
+  // (shock, fan head, fan tail, inside the fan) is chosen by selects, since it varies within a warp and a branch
+  // per case would run every path.  Velocities of the upwind side are taken positive toward the face (su, |u*|),
+  // so that the wave speeds need no products with the side's sign.
+  __device__ __forceinline__ void sample(const SP<float>& s, const float a[4], const float b[4], float ust, float2 W,
+                                         float2 IW, float F[4]) const {
     const bool left = ust > 0.0f;
-    const float sgn = left ? 1.0f : -1.0f;
-    const float ro = left ? rl : rr, uo = left ? ul : ur, vo = left ? vl : vr, po = left ? pl : pr;
-    const float wo = left ? wl : wr;
-    const float ico = left ? icl : icr;
-    const float iwo = (left ? tl : tr) * ico;
-    const float iro = rcpa(ro);                       // 1/rho_o
-    const float irst = iro - (pst - po) * iwo * iwo;  // 1/rho*, Hugoniot
+    const float aust = fabsf(ust);
+    const float ro = left ? a[0] : b[0], su = left ? a[1] : -b[1], fv = left ? a[2] : b[2], po = left ? a[3] : b[3];
+    const float wo = left ? W.x : W.y, iwo = left ? IW.x : IW.y;
+    const float co = s.gamma * po * (left ? IC.x : IC.y);  // sound speed
+    const float iro = rcpa(ro);                            // 1/rho_o
+    const float irst = iro - (pst - po) * iwo * iwo;       // 1/rho*, Hugoniot
     const float rst = rcpa(irst);
     const bool shock = pst > po;
-    const float S = uo - sgn * wo * iro;                        // shock speed
-    const float SH = uo - sgn * (g * po * ico);                 // fan head u_o -+ c_o
-    const float ST = ust - sgn * M<float>::sq(g * pst * irst);  // fan tail u* -+ c*
-    const bool take_o = shock ? sgn * S >= 0.0f : sgn * SH >= 0.0f;
-    const bool take_star = shock ? !take_o : sgn * ST <= 0.0f;
-    fr = take_o ? ro : rst;
-    fu = take_o ? uo : ust;
-    fp = take_o ? po : pst;
-    fv = vo;
-    // transonic fans are rare: the interpolation runs only in warps that have one
-    const bool in_fan = !take_o && !take_star;
-    if (__any_sync(__activemask(), in_fan)) {
+    const float SH = su - (shock ? wo * iro : co);  // shock speed or fan head
+    const float cst2 = s.gamma * pst * irst;        // square of the star state's sound speed
+    const bool take_o = SH >= 0.0f;
+    float fr = take_o ? ro : rst, fu = take_o ? su : aust, fp = take_o ? po : pst;
+    if (!shock && !take_o && aust * aust > cst2) {  // inside a transonic fan: rare
+      const float ST = aust - M<float>::sq(cst2);   // fan tail u* -+ c*
       const float frac = SH * rcpa(SH - ST);
-      if (in_fan) {
-        fr = ro + frac * (rst - ro);
-        fu = uo + frac * (ust - uo);
-        fp = po + frac * (pst - po);
-      }
+      fr = ro + frac * (rst - ro);
+      fu = su + frac * (aust - su);
+      fp = po + frac * (pst - po);
+    }
+    face_flux(s, fr, left ? fu : -fu, fv, fp, F);
+  }
+};
+
+__device__ __forceinline__ void riemann(const SP<float>& s, const float qL[4], const float qR[4], float guess,
+                                        float F[4], int& iters, bool& conv, float* pstar_out = nullptr) {
+  TwoShockF r;
+  r.start(s, qL, qR, guess);
+  r.step(s);
+  iters = 1;
+  conv = r.small_step(s);
+  if (!conv) iters = r.finish(s, 1, conv);
+  float2 W, IW;
+  const float ust = r.ustar(s, W, IW);
+  // a face on the contact (u* = 0; whole warps of it in a fluid at rest) carries the star pressure alone
+  F[0] = F[2] = F[3] = 0.0f;
+  F[1] = r.pst;
+  if (ust != 0.0f) r.sample(s, qL, qR, ust, W, IW, F);
+  if (pstar_out) *pstar_out = r.pst;
+}
+
+// Two faces at once, so that their chains of dependent operations overlap: the fluxes of riemann(a, b) and
+// riemann(c, d) from the acoustic start.  more += the iterations past the first of the faces that count (n0, n1), nonconv += those that
+// did not converge.
+__device__ __forceinline__ void riemann_pair(const SP<float>& s, const float a[4], const float b[4], bool n0, float F[4],
+                                             const float c[4], const float d[4], bool n1, float G[4],
+                                             unsigned int& more, unsigned int& nonconv) {
+  TwoShockF r, q;
+  r.start(s, a, b, 0.0f);
+  q.start(s, c, d, 0.0f);
+  r.step(s);
+  q.step(s);
+  bool ok0 = r.small_step(s), ok1 = q.small_step(s);
+  if (!(ok0 && ok1)) {
+    if (!ok0) {
+      const int it = r.finish(s, 1, ok0);
+      if (n0) { more += it - 1; nonconv += ok0 ? 0 : 1; }
+    }
+    if (!ok1) {
+      const int it = q.finish(s, 1, ok1);
+      if (n1) { more += it - 1; nonconv += ok1 ? 0 : 1; }
     }
   }
-  face_flux(s, fr, fu, fv, fp, F);
-  if (pstar_out) *pstar_out = pst;
+  float2 W0, IW0, W1, IW1;
+  const float u0 = r.ustar(s, W0, IW0), u1 = q.ustar(s, W1, IW1);
+  F[0] = F[2] = F[3] = G[0] = G[2] = G[3] = 0.0f;
+  F[1] = r.pst;
+  G[1] = q.pst;
+  if (u0 != 0.0f || u1 != 0.0f) {  // with u* = 0 the sampling gives the same flux
+    r.sample(s, a, b, u0, W0, IW0, F);
+    q.sample(s, c, d, u1, W1, IW1, G);
+  }
 }
 
 // HLLC approximate Riemann solver (§3.2's alternative solver, after Toro 1997) in the face frame
@@ -1022,15 +1126,8 @@ __device__ __forceinline__ void cfl_value(const SP<R>& s, R U0, R U1, R U2, R U3
     const float ke = __fmul_rn(__fmul_rn(0.5f, rho), __fadd_rn(__fmul_rn(u, u), __fmul_rn(v, v)));
     const float e = __fsub_rn(U3, ke);
     if (!(U0 > 0.0f) || !(e > 0.0f)) flags |= STATUS_NEGATIVE;
-    float p;
-    if (ke > __fmul_rn(s.rec, U3)) {  // as cons_to_prim: recover e = E - rho |u|^2 / 2 in double
-      const double rd = (double)rho, ud = __ddiv_rn((double)U1, rd), vd = __ddiv_rn((double)U2, rd);
-      p = (float)__dmul_rn((double)s.gm1,
-                           __dsub_rn((double)U3, __dmul_rn(__dmul_rn(0.5, rd), __dadd_rn(__dmul_rn(ud, ud),
-                                                                                      __dmul_rn(vd, vd)))));
-    } else {
-      p = __fmul_rn(s.gm1, e);
-    }
+    float p = __fmul_rn(s.gm1, e);
+    if (ke > __fmul_rn(s.rec, U3)) p = recovered_pressure_f64(s.gm1, rho, U1, U2, U3);  // as cons_to_prim
     p = p < s.small_pres ? s.small_pres : p;
     const float c2 = __fmul_rn(__fmul_rn(s.gamma, p), ir);
     const float cs = __fmul_rn(c2, rsqa(c2));

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
         q[k] = a[0];
         ppm_edges<R>(a[-2 * st], a[-st], a[0], a[st], a[2 * st], xi, eL[k], eR[k]);
       }
-      trace_ppm<R>(s, sigma, q, eL, eR, ql, qr);
+      trace_ppm<R>(s, sigma, q, eL, eR, Waves<R>(s, q[0], q[3]), ql, qr);
     } else {
       R dq[4];
 #pragma unroll
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
         q[k] = a[0];
         dq[k] = xi * slope<R>(s.limiter, a[-2 * st], a[-st], a[0], a[st], a[2 * st]);
       }
-      trace<R>(s, sigma, q, dq, ql, qr);
+      trace<R>(s, sigma, q, dq, Waves<R>(s, q[0], q[3]), ql, qr);
     }
     if (P.use_grav) {  // half-step gravity on v: transverse in the x sweep, normal in the y sweep
       constexpr int kv = DIR == 0 ? 2 : 1;
@@ -307,44 +307,9 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
       }
     }
   }
-  flush_counters<NT>(cnt, scr);
+  flush_counters(cnt, scr);
   if constexpr (FUSED) {
-    // block minimum of the CFL constraint; the last block to finish advances the time by this step's dt
-    // and writes the next step's factors (dt = cfl * min, clamped to reach tmax when tmax > 0)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const R o = __shfl_xor_sync(0xffffffffu, cmin, off);
-      cmin = M<R>::mnp(o, cmin);
-    }
-    __shared__ R wmin[NT / 32];
-    __shared__ bool last;
-    if ((tid & 31) == 0) wmin[tid >> 5] = cmin;
-    __syncthreads();
-    if (tid == 0) {
-      R b = wmin[0];
-      for (int k = 1; k < NT / 32; ++k) b = wmin[k] < b ? wmin[k] : b;
-      atomicMin(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong((double)b));
-      __threadfence();
-      last = atomicAdd(&scr->step_blocks_done, 1u) == gridDim.x * gridDim.y - 1u;
-    }
-    __syncthreads();
-    if (last && tid == 0) {
-      __threadfence();
-      const unsigned long long bits =
-          atomicExch(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong(DBL_MAX));
-      const double t = scr->t + sc.dt;
-      scr->t = t;
-      scr->nsteps = scr->nsteps + 1;
-      double dt = P.cfl * __longlong_as_double((long long)bits);
-      if (tmax > 0.0) {
-        const double left = tmax - t;
-        dt = dt > left ? left : dt;
-        dt = dt < 0.0 ? 0.0 : dt;
-      }
-      scr->dt = dt;
-      *sc_next = make_step_scalars(dt, P.dx, P.dy, P.grav);
-      scr->step_blocks_done = 0u;
-    }
+    finish_fused_step(P, cmin, &sc, sc_next, scr, tmax, 1u, gridDim.x * gridDim.y);
   }
 }
 
