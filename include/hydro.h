@@ -211,7 +211,7 @@ hydro_status hydro_step_host(hydro_ctx* ctx, const void* host_in, void* host_out
  * tmax and no other call that steps or replaces the state in between, this step's CFL time step is the
  * one the previous step reduced from the state it wrote (as hydro_step_fused keeps it), so no reduction
  * waits for the whole upload: each band of tile rows starts as soon as its rows and their 4-row halo
- * have arrived (eight bands), and the upload overlaps the step.  Otherwise the same as hydro_step_host.  The caller
+ * have arrived (five bands, eight above 2^21 cells), and the upload overlaps the step.  Otherwise the same as hydro_step_host.  The caller
  * must not modify host_out between the calls (the library checks the pointer, not the contents).  Same
  * results as hydro_step_host. */
 hydro_status hydro_step_host_chained(hydro_ctx* ctx, const void* host_in, void* host_out, double tmax);
@@ -384,12 +384,12 @@ const char* hydro_build_info(void);
 
 /* 1 if the context's step kernels load tiles by TMA bulk tensor copies (FP32 contexts with ng a multiple of
  * 4 on a driver that provides the tensor-map encoder; tiles whose halo leaves the interior, or the padded
- * array for the unfused step, are still loaded cell by cell), 0 otherwise or if ctx is NULL.  No paper
+ * array for the unfused step, and the strips that larger grids run in are still loaded cell by cell), 0 otherwise or if ctx is NULL.  No paper
  * counterpart: how the data reaches shared memory does not change what a step computes. */
 int hydro_tma_enabled(const hydro_ctx* ctx);
 
-/* Failure-path test of the bounded device-side wait (no paper counterpart).  drop = 1: the step kernels
- * issue no TMA tile copy, so each such tile's mbarrier waits for bytes that never arrive; the wait gives up
+/* Failure-path test of the bounded device-side wait (no paper counterpart).  drop = 1: the step runs in tiles
+ * whatever the grid, and the step kernels issue no TMA tile copy, so each such tile's mbarrier waits for bytes that never arrive; the wait gives up
  * after `polls` polls (1000 if 0), the tile is left unwritten and the status word records a timeout
  * (HYDRO_ETIMEOUT from hydro_sync_status).  Nothing is in flight when a tile gives up, and the context
  * stays usable.  drop = 0 restores normal operation.  Returns HYDRO_EINVAL for other values of drop. */

@@ -713,14 +713,17 @@ static cudaError_t enqueue_host_step(hydro_ctx* c, const void* host_in, void* ho
   // bands of tile rows, in sixteenths: 1/8, 1/8, 1/4, 1/4, 1/4 when every band waits for the dt (small
   // first bands start the copies back early); when chained, eight bands of 1/16, 1/8, 1/8, 3/16, 3/16, 1/8,
   // 1/8, 1/16 (a small first band starts the copies back early, a small last one ends the step early after
-  // the whole upload; KH 1024^2 FP32: 181 us per step, 186 us with 1/8, 1/4, 1/4, 1/4, 1/8, 185-200 us with
-  // five other splits); grids of fewer than 16 tile rows split evenly into at most five bands
+  // the whole upload), or up to 2^21 cells five bands of 3/16, 3/16, 1/4, 1/4, 1/8, since a band takes some 20 us
+  // however small it is (FP32, us per step with eight / five bands: KH 1024^2 194 / 188, 4096^2 2050 / 2156); grids
+  // of fewer than 16 tile rows split evenly into at most five bands
   static const int sixteenths_dt[6] = {0, 2, 4, 8, 12, 16};
   static const int sixteenths_chain[NB + 1] = {0, 1, 3, 5, 8, 11, 13, 15, 16};
+  static const int sixteenths_few[6] = {0, 3, 6, 10, 14, 16};
+  const bool few = (long long)ks.nx * ks.ny <= (1ll << 21);
   const int ty = hydro::fused_tile_rows(prec, c->kp);
   const int tile_h = hydro::fused_tile_height(prec);  // cells per tile row
-  const int nb = ty < 16 ? (ty < 5 ? ty : 5) : chained ? NB : 5;
-  const int* sixteenths = chained ? sixteenths_chain : sixteenths_dt;
+  const int nb = ty < 16 ? (ty < 5 ? ty : 5) : chained && !few ? NB : 5;
+  const int* sixteenths = !chained ? sixteenths_dt : few ? sixteenths_few : sixteenths_chain;
   int yb[NB + 1];
   for (int b = 0; b <= nb; ++b) yb[b] = ty >= 16 ? ty * sixteenths[b] / 16 : b * ty / nb;
   auto rows_up = [&](int r0, int r1) -> cudaError_t {  // padded rows [r0, r1) of the four planes
@@ -872,7 +875,7 @@ const char* hydro_last_error(const hydro_ctx* c) { return c ? c->err : "no conte
 
 const char* hydro_build_info(void) {
   return "hydro sm_103a; kernels: fill_ghost, cfl_dt, ctu_step and ctu_step_fused (fp64 16x16/384 or 16x8/384 exact rounding, "
-         "fp32 32x16/384 with TMA tile loads), batch fill/dt/step, totals, mlp";
+         "fp32 32x16/384 with TMA tile loads), march_step and march_step_fused (fp32 strips), batch fill/dt/step, totals, mlp";
 }
 
 int hydro_tma_enabled(const hydro_ctx* c) { return c ? c->tma_ok : 0; }

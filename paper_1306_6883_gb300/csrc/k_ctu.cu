@@ -1,5 +1,6 @@
-// Single-problem CTU step: the FP32 instantiations and the precision dispatch (FP64 in k_ctu_f64.cu).
-#include "ctu_kernels.cuh"
+// Single-problem CTU step: the FP32 instantiations (strips or tiles, march_kernels.cuh) and the precision dispatch
+// (FP64 in k_ctu_f64.cu).
+#include "march_kernels.cuh"
 
 namespace hydro {
 
@@ -9,21 +10,26 @@ int f32_tile_y() { return F32_TY; }
 cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, void* Uout, const StepScalars* sc_cur,
                            StepScalars* sc_next, DevScratch* scr, double tmax, const CUtensorMap* tmap,
                            cudaStream_t stream, int2 band, const MlpBlob* mlp) {
-  if (mlp != nullptr) {
-    // 320 threads (64 registers at 3 CTAs per SM): at 384 threads (56 registers) the gate test in the face
-    // loops, together with the pass over the queued faces, makes the allocator spill inside the loops
-    if (precision == 0 || P.reconstruction == 1 || P.riemann_solver == 1) return cudaErrorInvalidValue;
-    return launch_ctu_step_fused<float, F32_TX, F32_TY, 320, FACE_LEARNED>(
-        P, (const float*)Uin, (float*)Uout, sc_cur, sc_next, scr, tmax, tmap, stream, band, mlp);
-  }
+  if (mlp != nullptr && (precision == 0 || P.reconstruction == 1 || P.riemann_solver == 1)) return cudaErrorInvalidValue;
   if (P.reconstruction == 1)
     return ctu_step_fused_ppm(precision, P, Uin, Uout, sc_cur, sc_next, scr, tmax, tmap, stream, band);
   if (P.riemann_solver == 1)
     return ctu_step_fused_hllc(precision, P, Uin, Uout, sc_cur, sc_next, scr, tmax, tmap, stream, band);
   if (precision == 0)
     return ctu_step_fused_f64(P, (const double*)Uin, (double*)Uout, sc_cur, sc_next, scr, tmax, stream, band);
-  return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT>(P, (const float*)Uin, (float*)Uout, sc_cur, sc_next, scr,
-                                                              tmax, tmap, stream, band);
+  const float* in = (const float*)Uin;
+  float* out = (float*)Uout;
+  StripShape sh;
+  const cudaError_t e = choose_strips(P, &sh);
+  if (e != cudaSuccess) return e;
+  if (mlp != nullptr) {
+    // 320 threads (64 registers at 3 CTAs per SM): at 384 threads (56 registers) the gate test in the face
+    // loops, together with the pass over the queued faces, makes the allocator spill inside the loops
+    return launch_ctu_step_fused<float, F32_TX, F32_TY, 320, FACE_LEARNED>(P, in, out, sc_cur, sc_next, scr, tmax, tmap,
+                                                                           stream, band, mlp);
+  }
+  if (sh.nh) return launch_march_step_fused<FACE_PLAIN>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream, band);
+  return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band);
 }
 
 int fused_tile_height(int precision) { return precision == 0 ? F64_TY : F32_TY; }
@@ -42,6 +48,12 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
   const FaceHook h = hook ? *hook : FaceHook{};
   const float* in = (const float*)Uin;
   float* out = (float*)Uout;
+  StripShape sh{0, 0, 0};
+  if (mode != FACE_HARVEST) {  // the harvest samples faces by their place in a tile
+    const cudaError_t e = choose_strips(P, &sh);
+    if (e != cudaSuccess) return e;
+  }
+  if (sh.nh && mode != FACE_LEARNED) return launch_march_step<FACE_PLAIN>(sh, P, in, out, sc_host, sc_dev, scr, stream);
   switch (mode) {
     case FACE_HARVEST:
       return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_HARVEST>(P, in, out, sc_host, sc_dev, scr, h, tmap,

@@ -1,6 +1,6 @@
 // Single-problem CTU step with piecewise-parabolic reconstruction (RECON_PPM), with either Riemann solver:
 // the FP32 instantiations and the precision dispatch (FP64 in k_ctu_ppm_f64.cu).
-#include "ctu_kernels.cuh"
+#include "march_kernels.cuh"
 
 namespace hydro {
 
@@ -9,6 +9,13 @@ cudaError_t ctu_step_ppm(int precision, const KParams& P, const void* Uin, void*
   if (precision == 0) return ctu_step_ppm_f64(P, (const double*)Uin, (double*)Uout, sc_host, sc_dev, scr, stream);
   const float* in = (const float*)Uin;
   float* out = (float*)Uout;
+  StripShape sh;
+  const cudaError_t e = choose_strips(P, &sh);
+  if (e != cudaSuccess) return e;
+  if (sh.nh)
+    return P.riemann_solver == 1
+               ? launch_march_step<RECON_PPM | FACE_HLLC>(sh, P, in, out, sc_host, sc_dev, scr, stream)
+               : launch_march_step<RECON_PPM | FACE_PLAIN>(sh, P, in, out, sc_host, sc_dev, scr, stream);
   if (P.riemann_solver == 1)
     return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_HLLC>(P, in, out, sc_host, sc_dev, scr,
                                                                                  FaceHook{}, tmap, stream);
@@ -23,6 +30,14 @@ cudaError_t ctu_step_fused_ppm(int precision, const KParams& P, const void* Uin,
     return ctu_step_fused_ppm_f64(P, (const double*)Uin, (double*)Uout, sc_cur, sc_next, scr, tmax, stream, band);
   const float* in = (const float*)Uin;
   float* out = (float*)Uout;
+  StripShape sh;
+  const cudaError_t e = choose_strips(P, &sh);
+  if (e != cudaSuccess) return e;
+  if (sh.nh)
+    return P.riemann_solver == 1
+               ? launch_march_step_fused<RECON_PPM | FACE_HLLC>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream, band)
+               : launch_march_step_fused<RECON_PPM | FACE_PLAIN>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream,
+                                                                 band);
   if (P.riemann_solver == 1)
     return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_HLLC>(P, in, out, sc_cur, sc_next,
                                                                                        scr, tmax, tmap, stream, band);
