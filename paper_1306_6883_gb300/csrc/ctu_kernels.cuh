@@ -50,8 +50,8 @@ __device__ __forceinline__ void flush_counters(TileCounters& cnt, DevScratch* sc
 
 // End of a fused step for one block: its CFL minimum into the step's accumulator and its share into the step's
 // count; the block that completes the count (total) advances the time by this step's dt and writes the next step's
-// factors.
-template <typename R>
+// factors.  LAST false: the count is left to a later launch of the step.
+template <bool LAST = true, typename R>
 __device__ __forceinline__ void finish_fused_step(const KParams& P, R cmin, const StepScalars* sc_cur,
                                                   StepScalars* sc_next, DevScratch* scr, double tmax,
                                                   unsigned int share, unsigned int total) {
@@ -69,10 +69,10 @@ __device__ __forceinline__ void finish_fused_step(const KParams& P, R cmin, cons
     for (int k = 1; k < (int)(blockDim.x >> 5); ++k) b = wmin[k] < b ? wmin[k] : b;
     atomicMin(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong((double)b));
     __threadfence();
-    last = atomicAdd(&scr->step_blocks_done, share) + share == total;
+    last = LAST && atomicAdd(&scr->step_blocks_done, share) + share == total;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (LAST && last && threadIdx.x == 0) {
     __threadfence();
     const unsigned long long bits =
         atomicExch(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong(DBL_MAX));

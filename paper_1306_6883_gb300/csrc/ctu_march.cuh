@@ -66,13 +66,26 @@ __device__ __forceinline__ void face_pair(const SP<float>& s, const float a[4], 
   }
 }
 
+// Whether one of two counting faces is past the gate of the network mlp.
+__device__ __forceinline__ bool strong_pair(const MlpBlob* mlp, const float a[4], const float b[4], bool n0,
+                                            const float c[4], const float d[4], bool n1) {
+  const float ratio = __ldg(&mlp->gate_ratio), u4 = __ldg(&mlp->gate_u4);
+  return (n0 && strong_face(a, b, ratio, u4)) || (n1 && strong_face(c, d, ratio, u4));
+}
+
 // Steps the strip of nv columns (nv + 8 <= blockDim.x) and nh rows whose first interior cell is (i0, j0), padded
-// indices; smem holds march_bytes(blockDim.x).  MODE, FUSED, cfl_min as for ctu_tile.
+// indices; smem holds march_bytes(blockDim.x).  MODE, FUSED, cfl_min as for ctu_tile.  FACE_LEARNED: the strip solves
+// from the acoustic start and gives up (returns true, its rows then partly written) after the row in which a face
+// is past the gate of mlp; its tiles are then to be stepped with the network.  Such faces are few and lie together, and
+// a network pass in a strip would hold up all its later rows (a blast's front kept strips for 1 ms).
 template <int MODE, bool FUSED>
-__device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, const StepFactors<float>& f,
+__device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, const StepFactors<float>& f,
                                           const float* __restrict__ Uin, float* __restrict__ Uout, int i0, int nv, int j0,
-                                          int nh, unsigned char* smem, TileCounters& cnt, float* cfl_min = nullptr) {
-  static_assert(face_kind(MODE) == FACE_PLAIN || face_kind(MODE) == FACE_HLLC, "strips solve plain or HLLC faces");
+                                          int nh, unsigned char* smem, TileCounters& cnt, const MlpBlob* mlp,
+                                          float* cfl_min = nullptr) {
+  static_assert(face_kind(MODE) != FACE_HARVEST, "the harvest steps in tiles");
+  constexpr bool GATED = face_kind(MODE) == FACE_LEARNED;
+  bool strong = false;
   const int W = blockDim.x, x = threadIdx.x;  // column of the strip, its halo and copies of the last column past it
   const int xl1 = x > 0 ? x - 1 : 0, xr1 = x < W - 1 ? x + 1 : W - 1;
   float4* const ring_q = reinterpret_cast<float4*>(smem);
@@ -258,6 +271,7 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
     {
       float a[4], F[4];
       q_ld(x_l, xl1, a);
+      if constexpr (GATED) strong |= strong_pair(mlp, a, xr, on_xface, yl_c, yr, on_trace && c >= j0);
       face_pair<MODE>(s, a, xr, on_xface, fxh, yl_c, yr, on_trace && c >= j0, F, cnt);
       q_st(x_hat, x, fxh);
       const float G[4] = {F[0], F[2], F[1], F[3]};
@@ -287,6 +301,7 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
       ylc_new[0] = a[0]; ylc_new[1] = a[2]; ylc_new[2] = a[1]; ylc_new[3] = a[3];
       q_ld(x_lc, xl1, lc);
       float F[4];
+      if constexpr (GATED) strong |= strong_pair(mlp, ylc, yrc, on_cell && c >= j0, lc, xr_c, on_xface && c > j0);
       face_pair<MODE>(s, ylc, yrc, on_cell && c >= j0, F, lc, xr_c, on_xface && c > j0, gx, cnt);
       gy[0] = F[0]; gy[1] = F[2]; gy[2] = F[1]; gy[3] = F[3];
       q_ld(ring_u + sm * W, x, um);
@@ -313,7 +328,11 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
       ddu_c = ddu;
       ddv_c = ddv;
     }
-    __syncthreads();
+    if constexpr (GATED) {
+      if (__syncthreads_or(strong)) return true;
+    } else {
+      __syncthreads();
+    }
     // ---- update of row c - 1
     if (c > j0 && on_cell) {
       float fx1[4], Un[4];
@@ -350,6 +369,7 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
   const unsigned int solves = (on_xface ? 2 * nh + 2 : 0) + (on_trace ? nh + 1 : 0) + (on_cell ? nh + 1 : 0);
   cnt.solves += solves;
   if (face_kind(MODE) != FACE_HLLC) cnt.iters += solves;
+  return false;
 }
 
 }  // namespace hydro

@@ -318,6 +318,11 @@ hydro_status hydro_init(const hydro_params* p, void* d_state, void* d_state_alt,
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->partials, sizeof(double) * 4 * hydro::totals_max_blocks());
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->host_scr, sizeof(DevScratch));
   if (e == cudaSuccess) e = hydro::init_scratch(c->scr, c->stream);
+  if (p->use_learned_guess == 1) {
+    const size_t n = hydro::learned_work_bytes(c->kp);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&c->hook.learned_work, n);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->hook.learned_work, 0, n, c->stream);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     hydro_destroy(c);
@@ -347,6 +352,7 @@ void hydro_destroy(hydro_ctx* c) {
   }
   if (c->scr) cudaFree(c->scr);
   if (c->partials) cudaFree(c->partials);
+  if (c->hook.learned_work) cudaFree(c->hook.learned_work);
   if (c->host_scr) cudaFreeHost(c->host_scr);
   delete c;
 }
@@ -484,7 +490,8 @@ hydro_status hydro_step_fused(hydro_ctx* c, double tmax) {
   if (e == cudaSuccess)
     e = hydro::ctu_step_fused(c->p.precision, c->kp, c->state[c->cur], c->state[1 - c->cur],
                               &c->scr->scf[c->fused_parity], &c->scr->scf[1 - c->fused_parity], c->scr, tmax,
-                              c->tma_ok ? &c->tmap[c->cur] : nullptr, c->stream, make_int2(0, 0), ctx_model(c));
+                              c->tma_ok ? &c->tmap[c->cur] : nullptr, c->stream, make_int2(0, 0), ctx_model(c),
+                              c->hook.learned_work);
   if (e != cudaSuccess) return cuda_fail(c, e, "step_fused");
   ++c->step_calls;
   c->cur = 1 - c->cur;
@@ -761,7 +768,7 @@ static cudaError_t enqueue_host_step(hydro_ctx* c, const void* host_in, void* ho
     if (e == cudaSuccess)
       e = hydro::ctu_step_fused(prec, ks, s_in, s_out, sc_cur, sc_next, c->scr, tmax,
                                 c->stage_tma ? &c->stage_map : nullptr, bs, make_int2(yb[b], yb[b + 1] - yb[b]),
-                                ctx_model(c));
+                                ctx_model(c), c->hook.learned_work);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_band[b], bs);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->d2h_stream, c->ev_band[b], 0);
     // the band's padded rows in the four planes (the first and last bands also carry the ghost rows below

@@ -28,10 +28,14 @@ cudaError_t cfl_dt(int precision, const KParams& P, const void* U, DevScratch* s
 // band (optional): tile rows [band.x, band.x + band.y) only (band.y <= 0: the whole step); bands of one
 // step may run concurrently, the last tile of all of them finishes the step.  fused_tile_rows: the step's
 // number of tile rows for the precision.  mlp (FP32 piecewise-linear two-shock steps only, may be NULL):
-// start the Riemann iterations from the learned proposal of these weights (FACE_LEARNED).
+// start the Riemann iterations from the learned proposal of these weights (FACE_LEARNED).  learned_work: their work area
+// (learned_work_bytes of device memory, zeroed before its first use; the launches leave it zero), without which
+// learned steps run in tiles.
 cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, void* Uout, const StepScalars* sc_cur,
                            StepScalars* sc_next, DevScratch* scr, double tmax, const CUtensorMap* tmap,
-                           cudaStream_t stream, int2 band = make_int2(0, 0), const MlpBlob* mlp = nullptr);
+                           cudaStream_t stream, int2 band = make_int2(0, 0), const MlpBlob* mlp = nullptr,
+                           unsigned int* learned_work = nullptr);
+size_t learned_work_bytes(const KParams& P);
 int fused_tile_rows(int precision, const KParams& P);
 int fused_tile_height(int precision);
 

@@ -9,7 +9,7 @@ int f32_tile_y() { return F32_TY; }
 
 cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, void* Uout, const StepScalars* sc_cur,
                            StepScalars* sc_next, DevScratch* scr, double tmax, const CUtensorMap* tmap,
-                           cudaStream_t stream, int2 band, const MlpBlob* mlp) {
+                           cudaStream_t stream, int2 band, const MlpBlob* mlp, unsigned int* learned_work) {
   if (mlp != nullptr && (precision == 0 || P.reconstruction == 1 || P.riemann_solver == 1)) return cudaErrorInvalidValue;
   if (P.reconstruction == 1)
     return ctu_step_fused_ppm(precision, P, Uin, Uout, sc_cur, sc_next, scr, tmax, tmap, stream, band);
@@ -23,6 +23,13 @@ cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, voi
   const cudaError_t e = choose_strips(P, &sh);
   if (e != cudaSuccess) return e;
   if (mlp != nullptr) {
+    if (sh.nh && learned_work) {
+      const cudaError_t el = launch_march_step_fused<FACE_LEARNED>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream,
+                                                                   band, mlp, learned_work);
+      if (el != cudaSuccess) return el;
+      return launch_learned_tiles<true>(P, in, out, StepScalars{}, sc_cur, sc_next, scr, tmax, tmap, stream, band, mlp,
+                                        learned_work);
+    }
     // 320 threads (64 registers at 3 CTAs per SM): at 384 threads (56 registers) the gate test in the face
     // loops, together with the pass over the queued faces, makes the allocator spill inside the loops
     return launch_ctu_step_fused<float, F32_TX, F32_TY, 320, FACE_LEARNED>(P, in, out, sc_cur, sc_next, scr, tmax, tmap,
@@ -53,6 +60,13 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
     const cudaError_t e = choose_strips(P, &sh);
     if (e != cudaSuccess) return e;
   }
+  if (sh.nh && mode == FACE_LEARNED && h.learned_work) {
+    const cudaError_t e = launch_march_step<FACE_LEARNED>(sh, P, in, out, sc_host, sc_dev, scr, stream, h.mlp,
+                                                          h.learned_work);
+    if (e != cudaSuccess) return e;
+    return launch_learned_tiles<false>(P, in, out, sc_host, sc_dev, nullptr, scr, 0.0, tmap, stream, make_int2(0, 0),
+                                       h.mlp, h.learned_work);
+  }
   if (sh.nh && mode != FACE_LEARNED) return launch_march_step<FACE_PLAIN>(sh, P, in, out, sc_host, sc_dev, scr, stream);
   switch (mode) {
     case FACE_HARVEST:
@@ -64,6 +78,11 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
     default:
       return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_PLAIN>(P, in, out, sc_host, sc_dev, scr, h, tmap, stream);
   }
+}
+
+size_t learned_work_bytes(const KParams& P) {
+  const size_t tx = (P.nx + F32_TX - 1) / F32_TX, ty = (P.ny + F32_TY - 1) / F32_TY;
+  return sizeof(unsigned int) * (4 * ty + 2 * tx * ty);
 }
 
 }  // namespace hydro

@@ -9,10 +9,41 @@ namespace hydro {
 // A strip's registers (128 a thread) let 512 threads share an SM: four strips of 128 columns.
 constexpr int MARCH_MAX_THREADS = 128, MARCH_SM_THREADS = 512;
 
+// Work area of a learned step: the 32x16 tiles of the strips that met a strong face.  For each tile row, four words of
+// which a launch uses those of its first row (the list's length, the next tile to take, the blocks that are done, -);
+// then the list, a band's part beginning at its first tile; then a mark for each tile.  All zero between steps.
+struct LearnedWork {
+  unsigned int* counters;
+  int* list;
+  unsigned int* mark;
+  int tx;
+  __device__ __forceinline__ LearnedWork(const KParams& P, unsigned int* w, int by0) {
+    tx = (P.nx + F32_TX - 1) / F32_TX;
+    const int ty = (P.ny + F32_TY - 1) / F32_TY;
+    counters = w + 4 * by0;
+    list = (int*)(w + 4 * ty) + (size_t)by0 * tx;
+    mark = w + 4 * ty + (size_t)tx * ty;
+  }
+};
+
+// Puts the tiles that overlap a strip's cells [i0, i0 + nv) x [j0, j0 + nh) on the list, each once.
+__device__ __forceinline__ void list_strip(const KParams& P, unsigned int* work, int by0, int i0, int nv, int j0,
+                                           int nh) {
+  const LearnedWork w(P, work, by0);
+  const int bx0 = (i0 - P.ng) / F32_TX, bx1 = (i0 - P.ng + nv - 1) / F32_TX;
+  const int r0 = (j0 - P.ng) / F32_TY, r1 = (j0 - P.ng + nh - 1) / F32_TY;
+  const int n = (bx1 - bx0 + 1) * (r1 - r0 + 1);
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const int t = (r0 + k / (bx1 - bx0 + 1)) * w.tx + bx0 + k % (bx1 - bx0 + 1);
+    if (atomicExch(&w.mark[t], 1u) == 0u) w.list[atomicAdd(&w.counters[0], 1u)] = t;
+  }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MAX_THREADS)
     march_step_kernel(KParams P, const float* __restrict__ Uin, float* __restrict__ Uout, StepScalars sc_host,
-                      const StepScalars* __restrict__ sc_dev, DevScratch* __restrict__ scr, int nv, int nh) {
+                      const StepScalars* __restrict__ sc_dev, DevScratch* __restrict__ scr, int nv, int nh,
+                      const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   SP<float> s;
   s.load(P);
@@ -20,8 +51,11 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
   f.load(sc_dev ? *sc_dev : sc_host);
   TileCounters cnt;
   const int i0 = P.ng + blockIdx.x * nv, j0 = P.ng + blockIdx.y * nh;
-  ctu_march<MODE, false>(P, s, f, Uin, Uout, i0, min(nv, P.ng + P.nx - i0), j0, min(nh, P.ng + P.ny - j0), smem_raw,
-                            cnt);
+  const int cols = min(nv, P.ng + P.nx - i0), n = min(nh, P.ng + P.ny - j0);
+  if (ctu_march<MODE, false>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, mlp)) {
+    cnt = TileCounters();  // the strip's tiles count instead
+    list_strip(P, work, 0, i0, cols, j0, n);
+  }
   flush_counters(cnt, scr);
 }
 
@@ -31,7 +65,8 @@ template <int MODE>
 __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MAX_THREADS)
     march_step_fused_kernel(KParams P, const float* __restrict__ Uin, float* __restrict__ Uout,
                             const StepScalars* __restrict__ sc_cur, StepScalars* __restrict__ sc_next,
-                            DevScratch* __restrict__ scr, double tmax, int row0, int rows, int nv, int nh) {
+                            DevScratch* __restrict__ scr, double tmax, int row0, int rows, int nv, int nh,
+                            const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   SP<float> s;
   s.load(P);
@@ -52,12 +87,57 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
         cfl_value(s, u[0], u[1], u[2], u[3], cmin, cnt.flags);
       }
     }
-  } else {
-    ctu_march<MODE, true>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, &cmin);
+  } else if (ctu_march<MODE, true>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, mlp, &cmin)) {
+    cnt = TileCounters();  // the strip's tiles count instead
+    cmin = FLT_MAX;
+    list_strip(P, work, row0 / F32_TY, i0, cols, j0, n);
   }
   flush_counters(cnt, scr);
-  // a strip counts its rows, so that the bands of a step may cut it into segments of their own height
-  finish_fused_step(P, cmin, sc_cur, sc_next, scr, tmax, (unsigned int)n, gridDim.x * (unsigned int)P.ny);
+  // a strip counts its rows, so that the bands of a step may cut it into segments of their own height; a learned step
+  // is finished by the launch over the listed tiles
+  finish_fused_step<face_kind(MODE) != FACE_LEARNED>(P, cmin, sc_cur, sc_next, scr, tmax, (unsigned int)n, gridDim.x * (unsigned int)P.ny);
+}
+
+// The listed tiles of a learned step, from the network's proposals (blocks take them from the list until it is empty),
+// and for a fused step its end.  by0, rows: the tile rows of the launch (a band of the step, or all).
+template <bool FUSED>
+__global__ void __launch_bounds__(320, 3)
+    learned_tiles_kernel(KParams P, const float* __restrict__ Uin, float* __restrict__ Uout, StepScalars sc_host,
+                         const StepScalars* __restrict__ sc_dev, StepScalars* __restrict__ sc_next,
+                         DevScratch* __restrict__ scr, double tmax, const __grid_constant__ CUtensorMap tmap, int use_tma,
+                         int by0, int rows, const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ int cur;
+  const LearnedWork w(P, work, by0);
+  TileCounters cnt;
+  float cmin = FLT_MAX;
+  const unsigned int n = *(volatile unsigned int*)&w.counters[0];
+  if (n > 0) {
+    SP<float> s;
+    s.load(P);
+    StepFactors<float> f;
+    f.load(sc_dev ? *sc_dev : sc_host);
+    while (true) {
+      if (threadIdx.x == 0) {
+        const unsigned int k = atomicAdd(&w.counters[1], 1u);
+        cur = k < n ? w.list[k] : -1;
+        if (cur >= 0) w.mark[cur] = 0u;
+      }
+      __syncthreads();
+      const int t = cur;
+      if (t < 0) break;
+      ctu_tile<float, F32_TX, F32_TY, 320, FACE_LEARNED, FUSED, true>(P, s, f, Uin, Uout, t % w.tx, t / w.tx, smem_raw,
+                                                                      cnt, FaceHook{}, mlp, &cmin,
+                                                                      use_tma ? &tmap : nullptr);
+      __syncthreads();  // the tile's last shared-memory reads finish before the next tile's loads
+    }
+  }
+  flush_counters(cnt, scr);
+  if constexpr (FUSED)
+    finish_fused_step(P, cmin, sc_dev, sc_next, scr, tmax, (unsigned int)rows,
+                      gridDim.x * (unsigned int)((P.ny + F32_TY - 1) / F32_TY));
+  if (threadIdx.x == 0 && atomicAdd(&w.counters[2], 1u) == gridDim.x - 1u)
+    w.counters[0] = w.counters[1] = w.counters[2] = 0u;
 }
 
 // Strips of a grid: nv columns and nh rows each, `threads` a block.  nh == 0: the grid is stepped in tiles.
@@ -115,13 +195,13 @@ inline cudaError_t choose_strips(const KParams& P, StripShape* shape) {
 template <int MODE>
 cudaError_t launch_march_step(const StripShape& sh, const KParams& P, const float* Uin, float* Uout,
                               const StepScalars& sc_host, const StepScalars* sc_dev, DevScratch* scr,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, const MlpBlob* mlp = nullptr, unsigned int* work = nullptr) {
   static std::atomic<unsigned long long> attr_done{0};
   const cudaError_t e = smem_attr_once(march_step_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
   if (e != cudaSuccess) return e;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (P.ny + sh.nh - 1) / sh.nh);
   march_step_kernel<MODE><<<grid, sh.threads, march_bytes(sh.threads), stream>>>(
-      P, Uin, Uout, sc_host, sc_dev, scr, sh.nv, sh.nh);
+      P, Uin, Uout, sc_host, sc_dev, scr, sh.nv, sh.nh, mlp, work);
   return cudaGetLastError();
 }
 
@@ -131,7 +211,8 @@ cudaError_t launch_march_step(const StripShape& sh, const KParams& P, const floa
 template <int MODE>
 cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, const float* Uin, float* Uout,
                                     const StepScalars* sc_cur, StepScalars* sc_next, DevScratch* scr, double tmax,
-                                    cudaStream_t stream, int2 band) {
+                                    cudaStream_t stream, int2 band, const MlpBlob* mlp = nullptr,
+                                    unsigned int* work = nullptr) {
   static std::atomic<unsigned long long> attr_done{0};
   const cudaError_t e =
       smem_attr_once(march_step_fused_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
@@ -142,7 +223,27 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
   march_step_fused_kernel<MODE><<<grid, sh.threads, march_bytes(sh.threads), stream>>>(
-      P, Uin, Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh);
+      P, Uin, Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
+  return cudaGetLastError();
+}
+
+// A learned step of a grid that runs in strips: the strips, then the tiles they listed (three to an SM).
+template <bool FUSED>
+cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout, const StepScalars& sc_host,
+                                 const StepScalars* sc_dev, StepScalars* sc_next, DevScratch* scr, double tmax,
+                                 const CUtensorMap* tmap, cudaStream_t stream, int2 band, const MlpBlob* mlp,
+                                 unsigned int* work) {
+  static std::atomic<unsigned long long> attr_done{0};
+  const size_t smem = TileLayout<float, F32_TX, F32_TY>::bytes;
+  cudaError_t e = smem_attr_once(learned_tiles_kernel<FUSED>, smem, attr_done);
+  int dev = 0, nsm = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
+  learned_tiles_kernel<FUSED><<<3 * nsm, 320, smem, stream>>>(P, Uin, Uout, sc_host, sc_dev, sc_next, scr, tmax,
+                                                             tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp,
+                                                             work);
   return cudaGetLastError();
 }
 

@@ -44,6 +44,7 @@ struct FaceHook {
   // faces past this gate (as MlpBlob::gate_ratio / gate_u4) are recorded whatever their hash; 0 = off
   float hgate_ratio, hgate_u4;
   const MlpBlob* mlp;    // learned proposal weights (device), or null
+  unsigned int* learned_work;  // work area of learned steps in strips (learned_work_bytes, zeroed), or null
 };
 
 // Tile modes: the face-solve variant in the low two bits, and RECON_PPM for piecewise-parabolic

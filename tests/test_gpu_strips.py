@@ -74,3 +74,43 @@ def test_strips_cut_into_bands_give_the_same_state(nx, ny):
     np.testing.assert_array_equal(a.interior(), b.interior())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("gate", [None, (0.0, 0.0), (40.0, 1e9)])  # default, every face past it, none
+def test_learned_strips_hand_their_strong_faces_to_tiles(gate):
+    # an untrained network: its proposals change where the iterations start, not what they converge to
+    import torch
+    from paper_1306_6883_gb300 import hydro as H
+    from paper_1306_6883_gb300.solver import Model, Solver, params_for
+    pr = hp.quad(1030, 700, seed=7)
+    po = oracle.params(pr.nx, pr.ny, bc=pr.bc)
+    m = Model(seed=3)
+    if gate:
+        m.set_gate(*gate)
+    host = [torch.from_numpy(np.ascontiguousarray(pr.U)).float().pin_memory() for _ in range(2)]
+    solvers = [Solver(params_for(pr, H.HYDRO_FP32, use_learned_guess=1), pr.U) for _ in range(3)]
+    for s in solvers:
+        H.hydro_set_riemann_model(s.ctx, m.m)
+    U = solvers[0].state_numpy().astype(np.float64)
+    solvers[0].step_fused()
+    solvers[1].step_host(host[0], host[1])  # bands
+    dt = solvers[0].time()[0]
+    solvers[2].fill_ghost()
+    solvers[2].step(dt)
+    oracle.fill_ghost(po, U)
+    oracle.step(po, U, dt)
+    ref = U[:, NG:-NG, NG:-NG]
+    scale = np.abs(ref).reshape(4, -1).max(axis=1)[:, None, None]
+    got = [s.interior() for s in solvers]
+    for s, g in zip(solvers, got):
+        st, stats = s.status()
+        assert st == 0 and stats[2] == 0
+        assert np.all(np.abs(g - ref) <= 2e-5 * scale)
+    np.testing.assert_array_equal(got[0], got[1])
+    # the work area is left ready for the next step
+    for _ in range(3):
+        solvers[0].step_fused()
+    assert solvers[0].status()[0] == 0 and solvers[0].time()[1] == 4
+    for s in solvers:
+        s.close()
+    m.close()
