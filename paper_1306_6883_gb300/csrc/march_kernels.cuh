@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
                             DevScratch* __restrict__ scr, double tmax, int row0, int rows, int nv, int nh,
                             const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  step_begin(Uin, sc_cur);
   SP<float> s;
   s.load(P);
   StepFactors<float> f;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(320, 3)
                          int by0, int rows, const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int cur;
+  step_begin(Uin, sc_dev);
   const LearnedWork w(P, work, by0);
   TileCounters cnt;
   float cmin = FLT_MAX;
@@ -222,9 +224,8 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
   const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 8;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
-  march_step_fused_kernel<MODE><<<grid, sh.threads, march_bytes(sh.threads), stream>>>(
-      P, Uin, Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
-  return cudaGetLastError();
+  return launch_step_kernel(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
+                            Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
 // A learned step of a grid that runs in strips: the strips, then the tiles they listed (three to an SM).
@@ -241,10 +242,8 @@ cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
-  learned_tiles_kernel<FUSED><<<3 * nsm, 320, smem, stream>>>(P, Uin, Uout, sc_host, sc_dev, sc_next, scr, tmax,
-                                                             tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp,
-                                                             work);
-  return cudaGetLastError();
+  return launch_step_kernel(learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host,
+                            sc_dev, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp, work);
 }
 
 }  // namespace hydro

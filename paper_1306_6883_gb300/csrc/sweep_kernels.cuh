@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
   constexpr int PQ = L::PQ, PC = L::PC, PF = L::PF, nQ = L::nQ, nC = L::nC, nF = L::nF;
   constexpr int kn = DIR == 0 ? 1 : 2, kt = DIR == 0 ? 2 : 1;  // normal / transverse momentum components
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  step_begin(Uin, sc_dev);
   R* sq = reinterpret_cast<R*>(smem_raw);  // [4][nQ] primitives, face frame
   R* sG = sq;                               // [4][nF] fluxes (conserved order), after stage 2
   R* sxi = sq + 4 * nQ;                     // [nC]
@@ -331,15 +332,14 @@ struct Sweep {
     if (sc_next) {
       e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, L::bytes, done_fused);
       if (e != cudaSuccess) return e;
-      sweep_kernel<R, DIR, LN, NL, NT, true, MODE><<<grid, NT, L::bytes, stream>>>(P, Uin, Uout, sc_host, sc_dev, scr,
-                                                                                  check_state, sc_next, tmax);
+      return launch_step_kernel(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+                                sc_host, sc_dev, scr, check_state, sc_next, tmax);
     } else {
       e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, L::bytes, done_plain);
       if (e != cudaSuccess) return e;
-      sweep_kernel<R, DIR, LN, NL, NT, false, MODE><<<grid, NT, L::bytes, stream>>>(P, Uin, Uout, sc_host, sc_dev, scr,
-                                                                                   check_state, nullptr, 0.0);
+      return launch_step_kernel(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+                                sc_host, sc_dev, scr, check_state, (StepScalars*)nullptr, 0.0);
     }
-    return cudaGetLastError();
   }
 };
 
