@@ -4,6 +4,7 @@
 #pragma once
 #include <float.h>
 
+#include <algorithm>
 #include <atomic>
 #include <utility>
 
@@ -148,40 +149,6 @@ __global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_kernel(KPara
   flush_counters(cnt, scr);
 }
 
-// Fused steps follow one another on a stream, one launch each.  Their kernels are launched so that the next one's
-// blocks may be placed as soon as every block of this one has begun, and wait there for its end (step_begin, the
-// kernel's first statement): the launch itself then overlaps the step before (RT 317x951 39.0 -> 37.0 us per step, the
-// two sweeps of a split KH 1030x770 step 58.3 -> 53.9, HLLC KH 1024^2 60.4 -> 57.9).
-//
-// The pointers to what the step before wrote pass through the wait: a load through a const __restrict__ parameter
-// counts as one of data that does not change while the kernel runs, which a memory clobber does not hold back (the
-// step's factors were read ahead of the wait).
-template <typename State, typename Scalars>
-__device__ __forceinline__ void step_begin(State& Uin, Scalars& sc) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" : "+l"(Uin), "+l"(sc) : : "memory");
-}
-
-template <typename... Params, typename... Args>
-cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
-                               Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned int)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  // a captured step keeps plain dependencies: graphs that a program edits or queries see the edges they always had
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
-  if (e != cudaSuccess) return e;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 // Raises a kernel's dynamic shared-memory limit once per device (function attributes belong to the device's
 // context); later calls on the same device only test a bit.  Devices beyond 63 set it on every call.
 template <typename K>
@@ -208,6 +175,62 @@ cudaError_t launch_ctu_step(const KParams& P, const R* Uin, R* Uout, const StepS
   ctu_step_kernel<R, TX, TY, NT, MODE><<<grid, NT, smem, stream>>>(P, Uin, Uout, sc_host, sc_dev, scr, hook,
                                                                     tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0);
   return cudaGetLastError();
+}
+
+// Fused steps follow one another on a stream, one launch each.  Their kernels are launched so that the next one's
+// blocks may be placed as soon as every block of this one has begun, and wait there for its end (step_begin, the
+// kernel's first statement): the launch itself then overlaps the step before (RT 317x951 39.0 -> 37.0 us per step, the
+// two sweeps of a split KH 1030x770 step 58.3 -> 53.9, HLLC KH 1024^2 60.4 -> 57.9).
+//
+// The pointers to what the step before wrote pass through the wait: a load through a const __restrict__ parameter
+// counts as one of data that does not change while the kernel runs, which a memory clobber does not hold back (the
+// step's factors were read ahead of the wait).
+template <typename State, typename Scalars>
+__device__ __forceinline__ void step_begin(State& Uin, Scalars& sc) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" : "+l"(Uin), "+l"(sc) : : "memory");
+}
+
+constexpr size_t SM_SMEM = 228 << 10, BLOCK_SMEM = 1 << 10;  // shared memory of an SM, and what a block takes beside its own
+constexpr size_t STEP_SMEM_MAX = SM_SMEM / 2 - BLOCK_SMEM + 128;  // the most launch_step_kernel asks for
+
+inline cudaError_t sm_count(int* nsm) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e == cudaSuccess ? cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
+// Launches a fused step's kernel (its shared-memory limit raised to STEP_SMEM_MAX).  Blocks placed ahead of time go
+// where there is room, several to an SM that has none of the step before, so a grid of c blocks per SM or fewer asks for
+// as much shared memory as keeps an SM at c blocks (FP64 192^2, 144 tiles of which an SM takes two: 127 us per step
+// without the overlap, 199 with it, 124.5 with it and one tile to an SM; FP32 384^2 20.9, 22.5, 18.3).
+// one_round: overlap only a grid of one block per SM or fewer (FP64, where a step with two tiles on some SMs loses
+// more than the launch: 224x192 204.6 us without, 208 with; 64^2 75.3 and 73.2).
+template <typename... Params, typename... Args>
+cudaError_t launch_step_kernel(bool one_round, void (*kernel)(Params...), dim3 grid, int threads, size_t smem,
+                               cudaStream_t stream, Args&&... args) {
+  // a captured step keeps plain dependencies: graphs that a program edits or queries see the edges they always had
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int nsm = 0;
+  cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+  if (e == cudaSuccess) e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  const unsigned long long c = ((unsigned long long)grid.x * grid.y + nsm - 1) / nsm;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned int)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone && (c == 1 || !one_round) ? 1 : 0;
+  if (cfg.numAttrs && c < 16) {
+    const size_t keep = (SM_SMEM / (c + 1) & ~(size_t)127) - BLOCK_SMEM + 128;  // c + 1 of these do not fit, c do
+    if (keep > smem) cfg.dynamicSmemBytes = keep;
+  }
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // Fused step: the tile reads ghost cells through the boundary map and folds the CFL constraint of its new
@@ -263,22 +286,21 @@ cudaError_t launch_ctu_step_fused(const KParams& P, const R* Uin, R* Uout, const
                                   cudaStream_t stream, int2 band = make_int2(0, 0), const MlpBlob* mlp = nullptr) {
   const size_t smem = TileLayout<R, TX, TY>::bytes;
   static std::atomic<unsigned long long> attr_done{0};
-  cudaError_t e = smem_attr_once(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, smem, attr_done);
+  cudaError_t e = smem_attr_once(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, std::max(smem, STEP_SMEM_MAX), attr_done);
   if (e != cudaSuccess) return e;
   const int tx = (P.nx + TX - 1) / TX, ty = (P.ny + TY - 1) / TY;
   const int y0 = band.y > 0 ? band.x : 0, ny = band.y > 0 ? band.y : ty;
   if (y0 < 0 || ny <= 0 || y0 + ny > ty) return cudaErrorInvalidValue;
   dim3 grid(tx, ny);
-  return launch_step_kernel(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin, Uout, sc_cur,
-                            sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
+  return launch_step_kernel(!is_f32<R>(), ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin,
+                            Uout, sc_cur, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
                             (unsigned int)tx * (unsigned int)ty, mlp);
 }
 
 // Whether an FP64 step takes 16x8 tiles instead of 16x16 ones (see F64_TY_SMALL).
 inline cudaError_t f64_small_tile(const KParams& P, bool* small) {
-  int dev = 0, nsm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   auto rounds = [&](int ty) {
     const long long n = (long long)((P.nx + F64_TX - 1) / F64_TX) * ((P.ny + ty - 1) / ty);

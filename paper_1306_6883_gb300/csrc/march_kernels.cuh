@@ -187,9 +187,8 @@ inline StripShape strip_shape(int nx, int ny, int nsm) {
 inline cudaError_t choose_strips(const KParams& P, StripShape* shape) {
   *shape = StripShape{0, 0, 0};
   if (P.tma_test_drop) return cudaSuccess;
-  int dev = 0, nsm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
   if (e == cudaSuccess) *shape = strip_shape(P.nx, P.ny, nsm);
   return e;
 }
@@ -217,14 +216,14 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
                                     unsigned int* work = nullptr) {
   static std::atomic<unsigned long long> attr_done{0};
   const cudaError_t e =
-      smem_attr_once(march_step_fused_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
+      smem_attr_once(march_step_fused_kernel<MODE>, std::max(march_bytes(MARCH_MAX_THREADS), STEP_SMEM_MAX), attr_done);
   if (e != cudaSuccess) return e;
   const int row0 = band.y > 0 ? band.x * F32_TY : 0;
   const int rows = band.y > 0 ? min(band.y * F32_TY, P.ny - row0) : P.ny;
   const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 8;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
-  return launch_step_kernel(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
+  return launch_step_kernel(false, march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
                             Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
@@ -236,13 +235,12 @@ cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout
                                  unsigned int* work) {
   static std::atomic<unsigned long long> attr_done{0};
   const size_t smem = TileLayout<float, F32_TX, F32_TY>::bytes;
-  cudaError_t e = smem_attr_once(learned_tiles_kernel<FUSED>, smem, attr_done);
-  int dev = 0, nsm = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = smem_attr_once(learned_tiles_kernel<FUSED>, std::max(smem, STEP_SMEM_MAX), attr_done);
+  int nsm = 0;
+  if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
-  return launch_step_kernel(learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host,
+  return launch_step_kernel(false, learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host,
                             sc_dev, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp, work);
 }
 
