@@ -113,6 +113,13 @@ constexpr int F32_TX = HYDRO_F32_TX, F32_TY = HYDRO_F32_TY, F32_NT = HYDRO_F32_N
 #ifndef HYDRO_F32_MINB
 #define HYDRO_F32_MINB 3
 #endif
+// The FP32 tile of grids so small that all its tiles run at once, three to an SM: such a step takes as long as one
+// block's chain of stages, which is shortest where each thread has one item per stage.  Measured per step, 16x8 at
+// 384 threads / 32x16 (KH, us): 64^2 9.3 / 15.1, 192^2 (two tiles an SM / one) 10.6 / 15.2, 224^2 (three / one) 11.8 /
+// 15.1, 256^2 (four, so two rounds / one) 14.9 / 15.2, 384^2 (eight / two) 23.9 / 18.3.  16x8 at 192 threads takes
+// 10.6 at 64^2 and 12.4 at 224^2, 32x8 at 384 11.7 and 13.5, 8x8 at 256 9.1 and 14.2 (five to an SM).
+constexpr int F32_SMALL_TX = 16, F32_SMALL_TY = 8;
+
 // Tiles of the FP64 kernels.  Their time is the SM's one FP64 unit, so a tile's cost is its FP64 instructions,
 // and what counts is the halo (for large grids) or how many SMs have a tile at all (for small ones).  Measured on
 // KH 1024^2 per step / Sod 128^2 host loop per step: 16x16 at 384 threads, two per SM 2.75 ms / 155 us; at 256
@@ -332,6 +339,45 @@ cudaError_t launch_ctu_step_fused_f64(const KParams& P, const double* Uin, doubl
   const auto launch = small ? launch_ctu_step_fused<double, F64_TX, F64_TY_SMALL, F64_NT, MODE>
                             : launch_ctu_step_fused<double, F64_TX, F64_TY, F64_NT, MODE>;
   return launch(P, Uin, Uout, sc_cur, sc_next, scr, tmax, nullptr, stream, band, nullptr);
+}
+
+// Whether an FP32 step in tiles takes the small ones (see F32_SMALL_TX).  The withheld-copy test
+// (hydro_test_drop_tile_copies) keeps the large ones, which load through the tensor map.
+inline cudaError_t f32_small_tile(const KParams& P, bool* small) {
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
+  const long long n =
+      (long long)((P.nx + F32_SMALL_TX - 1) / F32_SMALL_TX) * ((P.ny + F32_SMALL_TY - 1) / F32_SMALL_TY);
+  *small = !P.tma_test_drop && n <= (long long)HYDRO_F32_MINB * nsm;
+  return e;
+}
+
+template <int MODE, int NT = F32_NT>
+cudaError_t launch_ctu_step_f32(const KParams& P, const float* Uin, float* Uout, const StepScalars& sc_host,
+                                const StepScalars* sc_dev, DevScratch* scr, const FaceHook& hook,
+                                const CUtensorMap* tmap, cudaStream_t stream) {
+  bool small = false;
+  const cudaError_t e = f32_small_tile(P, &small);
+  if (e != cudaSuccess) return e;
+  if (small)
+    return launch_ctu_step<float, F32_SMALL_TX, F32_SMALL_TY, NT, MODE>(P, Uin, Uout, sc_host, sc_dev, scr, hook,
+                                                                        nullptr, stream);
+  return launch_ctu_step<float, F32_TX, F32_TY, NT, MODE>(P, Uin, Uout, sc_host, sc_dev, scr, hook, tmap, stream);
+}
+
+// A band of a step (band.y > 0) counts tile rows of F32_TY cells.
+template <int MODE, int NT = F32_NT>
+cudaError_t launch_ctu_step_fused_f32(const KParams& P, const float* Uin, float* Uout, const StepScalars* sc_cur,
+                                      StepScalars* sc_next, DevScratch* scr, double tmax, const CUtensorMap* tmap,
+                                      cudaStream_t stream, int2 band, const MlpBlob* mlp = nullptr) {
+  bool small = false;
+  const cudaError_t e = band.y > 0 ? cudaSuccess : f32_small_tile(P, &small);
+  if (e != cudaSuccess) return e;
+  if (small)
+    return launch_ctu_step_fused<float, F32_SMALL_TX, F32_SMALL_TY, NT, MODE>(P, Uin, Uout, sc_cur, sc_next, scr, tmax,
+                                                                              nullptr, stream, band, mlp);
+  return launch_ctu_step_fused<float, F32_TX, F32_TY, NT, MODE>(P, Uin, Uout, sc_cur, sc_next, scr, tmax, tmap, stream,
+                                                                band, mlp);
 }
 
 }  // namespace hydro

@@ -32,11 +32,10 @@ cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, voi
     }
     // 320 threads (64 registers at 3 CTAs per SM): at 384 threads (56 registers) the gate test in the face
     // loops, together with the pass over the queued faces, makes the allocator spill inside the loops
-    return launch_ctu_step_fused<float, F32_TX, F32_TY, 320, FACE_LEARNED>(P, in, out, sc_cur, sc_next, scr, tmax, tmap,
-                                                                           stream, band, mlp);
+    return launch_ctu_step_fused_f32<FACE_LEARNED, 320>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band, mlp);
   }
   if (sh.nh) return launch_march_step_fused<FACE_PLAIN>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream, band);
-  return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band);
+  return launch_ctu_step_fused_f32<FACE_PLAIN>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band);
 }
 
 int fused_tile_height(int precision) { return precision == 0 ? F64_TY : F32_TY; }
@@ -73,10 +72,9 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
       return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_HARVEST>(P, in, out, sc_host, sc_dev, scr, h, tmap,
                                                                            stream);
     case FACE_LEARNED:
-      return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_LEARNED>(P, in, out, sc_host, sc_dev, scr, h, tmap,
-                                                                           stream);
+      return launch_ctu_step_f32<FACE_LEARNED>(P, in, out, sc_host, sc_dev, scr, h, tmap, stream);
     default:
-      return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_PLAIN>(P, in, out, sc_host, sc_dev, scr, h, tmap, stream);
+      return launch_ctu_step_f32<FACE_PLAIN>(P, in, out, sc_host, sc_dev, scr, h, tmap, stream);
   }
 }
 

@@ -13,8 +13,7 @@ cudaError_t ctu_step_hllc(int precision, const KParams& P, const void* Uin, void
   if (e != cudaSuccess) return e;
   if (sh.nh)
     return launch_march_step<FACE_HLLC>(sh, P, (const float*)Uin, (float*)Uout, sc_host, sc_dev, scr, stream);
-  return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, FACE_HLLC>(P, (const float*)Uin, (float*)Uout, sc_host,
-                                                                    sc_dev, scr, FaceHook{}, tmap, stream);
+  return launch_ctu_step_f32<FACE_HLLC>(P, (const float*)Uin, (float*)Uout, sc_host, sc_dev, scr, FaceHook{}, tmap, stream);
 }
 
 cudaError_t ctu_step_fused_hllc(int precision, const KParams& P, const void* Uin, void* Uout,
@@ -28,8 +27,8 @@ cudaError_t ctu_step_fused_hllc(int precision, const KParams& P, const void* Uin
   if (sh.nh)
     return launch_march_step_fused<FACE_HLLC>(sh, P, (const float*)Uin, (float*)Uout, sc_cur, sc_next, scr, tmax, stream,
                                               band);
-  return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT, FACE_HLLC>(P, (const float*)Uin, (float*)Uout, sc_cur,
-                                                                          sc_next, scr, tmax, tmap, stream, band);
+  return launch_ctu_step_fused_f32<FACE_HLLC>(P, (const float*)Uin, (float*)Uout, sc_cur, sc_next, scr, tmax, tmap,
+                                              stream, band);
 }
 
 }  // namespace hydro

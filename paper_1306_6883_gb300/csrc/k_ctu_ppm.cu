@@ -17,10 +17,8 @@ cudaError_t ctu_step_ppm(int precision, const KParams& P, const void* Uin, void*
                ? launch_march_step<RECON_PPM | FACE_HLLC>(sh, P, in, out, sc_host, sc_dev, scr, stream)
                : launch_march_step<RECON_PPM | FACE_PLAIN>(sh, P, in, out, sc_host, sc_dev, scr, stream);
   if (P.riemann_solver == 1)
-    return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_HLLC>(P, in, out, sc_host, sc_dev, scr,
-                                                                                 FaceHook{}, tmap, stream);
-  return launch_ctu_step<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_PLAIN>(P, in, out, sc_host, sc_dev, scr,
-                                                                                FaceHook{}, tmap, stream);
+    return launch_ctu_step_f32<RECON_PPM | FACE_HLLC>(P, in, out, sc_host, sc_dev, scr, FaceHook{}, tmap, stream);
+  return launch_ctu_step_f32<RECON_PPM | FACE_PLAIN>(P, in, out, sc_host, sc_dev, scr, FaceHook{}, tmap, stream);
 }
 
 cudaError_t ctu_step_fused_ppm(int precision, const KParams& P, const void* Uin, void* Uout,
@@ -39,10 +37,8 @@ cudaError_t ctu_step_fused_ppm(int precision, const KParams& P, const void* Uin,
                : launch_march_step_fused<RECON_PPM | FACE_PLAIN>(sh, P, in, out, sc_cur, sc_next, scr, tmax, stream,
                                                                  band);
   if (P.riemann_solver == 1)
-    return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_HLLC>(P, in, out, sc_cur, sc_next,
-                                                                                       scr, tmax, tmap, stream, band);
-  return launch_ctu_step_fused<float, F32_TX, F32_TY, F32_NT, RECON_PPM | FACE_PLAIN>(P, in, out, sc_cur, sc_next,
-                                                                                      scr, tmax, tmap, stream, band);
+    return launch_ctu_step_fused_f32<RECON_PPM | FACE_HLLC>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band);
+  return launch_ctu_step_fused_f32<RECON_PPM | FACE_PLAIN>(P, in, out, sc_cur, sc_next, scr, tmax, tmap, stream, band);
 }
 
 }  // namespace hydro
