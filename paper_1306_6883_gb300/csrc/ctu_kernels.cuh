@@ -78,7 +78,7 @@ __device__ __forceinline__ void finish_fused_step(const KParams& P, R cmin, cons
     __threadfence();
     const unsigned long long bits =
         atomicExch(&scr->dtn_min_bits, (unsigned long long)__double_as_longlong(DBL_MAX));
-    const double t = scr->t + sc_cur->dt;
+    const double t = scr->t + ld_ordered(&sc_cur->dt);
     scr->t = t;
     scr->nsteps = scr->nsteps + 1;
     double dt = P.cfl * __longlong_as_double((long long)bits);
@@ -187,15 +187,11 @@ cudaError_t launch_ctu_step(const KParams& P, const R* Uin, R* Uout, const StepS
 // Fused steps follow one another on a stream, one launch each.  Their kernels are launched so that the next one's
 // blocks may be placed as soon as every block of this one has begun, and wait there for its end (step_begin, the
 // kernel's first statement): the launch itself then overlaps the step before (RT 317x951 39.0 -> 37.0 us per step, the
-// two sweeps of a split KH 1030x770 step 58.3 -> 53.9, HLLC KH 1024^2 60.4 -> 57.9).
-//
-// The pointers to what the step before wrote pass through the wait: a load through a const __restrict__ parameter
-// counts as one of data that does not change while the kernel runs, which a memory clobber does not hold back (the
-// step's factors were read ahead of the wait).
-template <typename State, typename Scalars>
-__device__ __forceinline__ void step_begin(State& Uin, Scalars& sc) {
+// two sweeps of a split KH 1030x770 step 58.3 -> 53.9, HLLC KH 1024^2 60.4 -> 57.9).  What the
+// step before wrote is read with ld_ordered.
+__device__ __forceinline__ void step_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" : "+l"(Uin), "+l"(sc) : : "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 constexpr size_t SM_SMEM = 228 << 10, BLOCK_SMEM = 1 << 10;  // shared memory of an SM, and what a block takes beside its own
@@ -211,11 +207,13 @@ inline cudaError_t sm_count(int* nsm) {
 // where there is room, several to an SM that has none of the step before, so a grid of c blocks per SM or fewer asks for
 // as much shared memory as keeps an SM at c blocks (FP64 192^2, 144 tiles of which an SM takes two: 127 us per step
 // without the overlap, 199 with it, 124.5 with it and one tile to an SM; FP32 384^2 20.9, 22.5, 18.3).
-// one_round: overlap only a grid of one block per SM or fewer (FP64, where a step with two tiles on some SMs loses
-// more than the launch: 224x192 204.6 us without, 208 with; 64^2 75.3 and 73.2).
-template <typename... Params, typename... Args>
-cudaError_t launch_step_kernel(bool one_round, void (*kernel)(Params...), dim3 grid, int threads, size_t smem,
-                               cudaStream_t stream, Args&&... args) {
+// Which steps overlap: in FP64 those of one block per SM or fewer, since a step with two tiles on some SMs loses more
+// than the launch (224x192 204.6 us without, 208 with; 64^2 75.3 and 73.2).  With the learned start, whose blocks differ
+// in cost, not those that fill some SMs' last places: SMs that are done early would take more than their share of the
+// next step (Sedov 400^2 38.6 us without, 40.2 with; 300^2 36.9 and 34.3).  Else all.
+template <typename R, int MODE, typename... Params, typename... Args>
+cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
+                               Args&&... args) {
   // a captured step keeps plain dependencies: graphs that a program edits or queries see the edges they always had
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   int nsm = 0;
@@ -232,7 +230,8 @@ cudaError_t launch_step_kernel(bool one_round, void (*kernel)(Params...), dim3 g
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = &attr;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone && (c == 1 || !one_round) ? 1 : 0;
+  const bool overlap = !is_f32<R>() ? c == 1 : face_kind(MODE) != FACE_LEARNED || c != HYDRO_F32_MINB;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone && overlap ? 1 : 0;
   if (cfg.numAttrs && c < 16) {
     const size_t keep = (SM_SMEM / (c + 1) & ~(size_t)127) - BLOCK_SMEM + 128;  // c + 1 of these do not fit, c do
     if (keep > smem) cfg.dynamicSmemBytes = keep;
@@ -254,17 +253,17 @@ __global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_fused_kernel
                                                             int by0, unsigned int nblocks,
                                                             const MlpBlob* __restrict__ mlp) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  step_begin(Uin, sc_cur);
+  step_begin();
   // FACE_LEARNED: the network's weights (read from global memory by the warps whose gate opens)
   const MlpBlob* wsm = face_kind(MODE) == FACE_LEARNED ? mlp : nullptr;
   SP<R> s;
   s.load(P);
   StepFactors<R> f;
-  f.load(*sc_cur);
+  f.load_ordered(sc_cur);
   TileCounters cnt;
   R cmin = is_f32<R>() ? (R)FLT_MAX : (R)DBL_MAX;
   const int by = by0 + (int)blockIdx.y;
-  if (sf_zero(sc_cur->dt)) {
+  if (sf_zero(ld_ordered(&sc_cur->dt))) {
     // a step of length zero (the run has reached tmax) leaves the state as it is: copy the tile's interior
     // cells and take their CFL constraint as a step would (the next dt is then clamped to 0 again)
     const size_t plane = (size_t)P.NY * P.pitch;
@@ -274,7 +273,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R, TY>()) ctu_step_fused_kernel
       const size_t o = (size_t)gj * P.pitch + gi;
       R u[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) Uout[o + k * plane] = u[k] = Uin[o + k * plane];
+      for (int k = 0; k < 4; ++k) Uout[o + k * plane] = u[k] = ld_ordered(Uin + o + k * plane);
       cfl_value(s, u[0], u[1], u[2], u[3], cmin, cnt.flags);
     }
   } else {
@@ -299,7 +298,7 @@ cudaError_t launch_ctu_step_fused(const KParams& P, const R* Uin, R* Uout, const
   const int y0 = band.y > 0 ? band.x : 0, ny = band.y > 0 ? band.y : ty;
   if (y0 < 0 || ny <= 0 || y0 + ny > ty) return cudaErrorInvalidValue;
   dim3 grid(tx, ny);
-  return launch_step_kernel(!is_f32<R>(), ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin,
+  return launch_step_kernel<R, MODE>(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin,
                             Uout, sc_cur, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
                             (unsigned int)tx * (unsigned int)ty, mlp);
 }

@@ -110,7 +110,7 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
     const int r = FUSED ? map_index(row, P.ng, P.ny, P.bc[2], P.bc[3]) : (row < P.NY ? row : P.NY - 1);
     const float* a = Uin + (size_t)r * P.pitch + col;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) u[k] = __ldg(a + k * plane);
+    for (int k = 0; k < 4; ++k) u[k] = ld_ordered(a + k * plane);
   };
   auto slot = [](int newest, int back) { return newest >= back ? newest - back : newest - back + MARCH_ROWS; };
   // a fetched row into ring slot sl; returns its primitives

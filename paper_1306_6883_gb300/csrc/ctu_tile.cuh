@@ -81,7 +81,7 @@ __device__ __forceinline__ void tile_cell(const KParams& P, const R* __restrict_
   } else {
     const size_t o = cell_offset<FUSED>(P, gi, gj);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = __ldg(U + o + k * plane);
+    for (int k = 0; k < 4; ++k) v[k] = ld_ordered(U + o + k * plane);
   }
 }
 
@@ -94,6 +94,16 @@ struct TileCounters {
 template <typename R>
 struct StepFactors {
   R sigx, sigy, hx, hy, hdtg;
+  // the factors that the step before wrote
+  __device__ __forceinline__ void load_ordered(const StepScalars* sc) {
+    if constexpr (is_f32<R>()) {
+      sigx = ld_ordered(&sc->sigx_f); sigy = ld_ordered(&sc->sigy_f);
+      hx = ld_ordered(&sc->hx_f); hy = ld_ordered(&sc->hy_f); hdtg = ld_ordered(&sc->hdtg_f);
+    } else {
+      sigx = ld_ordered(&sc->sigx); sigy = ld_ordered(&sc->sigy);
+      hx = ld_ordered(&sc->hx); hy = ld_ordered(&sc->hy); hdtg = ld_ordered(&sc->hdtg);
+    }
+  }
   __device__ __forceinline__ void load(const StepScalars& sc) {
     if constexpr (is_f32<R>()) {
       sigx = sc.sigx_f; sigy = sc.sigy_f; hx = sc.hx_f; hy = sc.hy_f; hdtg = sc.hdtg_f;
@@ -305,7 +315,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
           } else {
             const size_t o = cell_offset<FUSED>(P, gi, gj);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) Ul[it][k] = __ldg(Uin + o + k * plane);
+            for (int k = 0; k < 4; ++k) Ul[it][k] = ld_ordered(Uin + o + k * plane);
           }
         }
       }
@@ -710,7 +720,7 @@ __device__ __forceinline__ void ctu_tile(const KParams& P, const SP<R>& s, const
       Quad<R, nC>::ld(sU, cy + SX, un);  // the cell's own U^n, s index (ty + 1) * SX + tx + 1
     } else {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) un[k] = __ldg(Uin + o + k * plane);
+      for (int k = 0; k < 4; ++k) un[k] = ld_ordered(Uin + o + k * plane);
     }
     rho_n = un[0];
     my_n = un[2];

@@ -244,6 +244,20 @@ __device__ __forceinline__ int ghost_bc(int i, int ng, int n, int lo_bc, int hi_
   return i < ng ? lo_bc : i >= ng + n ? hi_bc : -1;
 }
 
+// A load of what an earlier kernel of the stream wrote, for kernels that start before that one has ended and wait for it
+// (step_begin).  A load through a const __restrict__ pointer, or __ldg, reads data that by contract does not change while
+// the kernel runs, and such a load may move ahead of the wait (the split step's factors did); this one may not.
+__device__ __forceinline__ float ld_ordered(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ double ld_ordered(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+
 // Value of the padded cell (i, j) as the ghost fill defines it (an interior cell: its stored value).  The
 // source is the interior cell (map_x(i), map_y(j)); a reflecting side negates the momentum normal to it (mx
 // across x walls, my across y walls).  A hydrostatic y side keeps the edge row's density and momenta and
@@ -258,7 +272,7 @@ __device__ __forceinline__ void bc_cell(const KParams& P, const R* U, int i, int
   const int sj = map_index(j, P.ng, P.ny, P.bc[2], P.bc[3]);
   const size_t s = (size_t)sj * P.pitch + si;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = U[s + k * plane];
+  for (int k = 0; k < 4; ++k) v[k] = ld_ordered(U + s + k * plane);
   if (ghost_bc(i, P.ng, P.nx, P.bc[0], P.bc[1]) == 2) v[1] = -v[1];
   const int ybc = ghost_bc(j, P.ng, P.ny, P.bc[2], P.bc[3]);
   if (ybc == 2) {

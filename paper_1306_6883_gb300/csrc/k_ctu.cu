@@ -20,7 +20,7 @@ cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, voi
   const float* in = (const float*)Uin;
   float* out = (float*)Uout;
   StripShape sh;
-  const cudaError_t e = choose_strips(P, &sh);
+  const cudaError_t e = choose_strips(P, &sh, mlp != nullptr);
   if (e != cudaSuccess) return e;
   if (mlp != nullptr) {
     if (sh.nh && learned_work) {
@@ -56,7 +56,7 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
   float* out = (float*)Uout;
   StripShape sh{0, 0, 0};
   if (mode != FACE_HARVEST) {  // the harvest samples faces by their place in a tile
-    const cudaError_t e = choose_strips(P, &sh);
+    const cudaError_t e = choose_strips(P, &sh, mode == FACE_LEARNED);
     if (e != cudaSuccess) return e;
   }
   if (sh.nh && mode == FACE_LEARNED && h.learned_work) {

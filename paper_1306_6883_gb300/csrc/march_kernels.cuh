@@ -68,23 +68,23 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
                             DevScratch* __restrict__ scr, double tmax, int row0, int rows, int nv, int nh,
                             const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  step_begin(Uin, sc_cur);
+  step_begin();
   SP<float> s;
   s.load(P);
   StepFactors<float> f;
-  f.load(*sc_cur);
+  f.load_ordered(sc_cur);
   TileCounters cnt;
   float cmin = FLT_MAX;
   const int i0 = P.ng + blockIdx.x * nv, j0 = P.ng + row0 + blockIdx.y * nh;
   const int cols = min(nv, P.ng + P.nx - i0), n = min(nh, P.ng + row0 + rows - j0);
-  if (sf_zero(sc_cur->dt)) {  // a step of length zero: copy (ctu_step_fused_kernel)
+  if (sf_zero(ld_ordered(&sc_cur->dt))) {  // a step of length zero: copy (ctu_step_fused_kernel)
     const size_t plane = (size_t)P.NY * P.pitch;
     if ((int)threadIdx.x < cols) {
       for (int j = 0; j < n; ++j) {
         const size_t o = (size_t)(j0 + j) * P.pitch + i0 + threadIdx.x;
         float u[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) Uout[o + k * plane] = u[k] = Uin[o + k * plane];
+        for (int k = 0; k < 4; ++k) Uout[o + k * plane] = u[k] = ld_ordered(Uin + o + k * plane);
         cfl_value(s, u[0], u[1], u[2], u[3], cmin, cnt.flags);
       }
     }
@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(320, 3)
                          int by0, int rows, const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int cur;
-  step_begin(Uin, sc_dev);
   const LearnedWork w(P, work, by0);
   TileCounters cnt;
   float cmin = FLT_MAX;
@@ -183,14 +182,20 @@ inline StripShape strip_shape(int nx, int ny, int nsm) {
 }
 
 // The shape for a launch (nh == 0: tiles).  The withheld-copy test (hydro_test_drop_tile_copies) steps in tiles,
-// whose loads it is about.
-inline cudaError_t choose_strips(const KParams& P, StripShape* shape) {
+// whose loads it is about.  A learned step's strips give up where they meet a strong face and cost a second launch, of
+// tiles three to an SM, so they need many waves of tiles to gain (us per step, tiles / strips, KH and quad problems:
+// 600x500 35.9 / 44.1 and 40.7 / 76.8, 1000^2 88 / 89 and 100 / 121, 1900^2 278 / 243 and 305 / 302).
+constexpr int LEARNED_STRIP_WAVES = 16;
+
+inline cudaError_t choose_strips(const KParams& P, StripShape* shape, bool learned = false) {
   *shape = StripShape{0, 0, 0};
   if (P.tma_test_drop) return cudaSuccess;
   int nsm = 0;
   const cudaError_t e = sm_count(&nsm);
-  if (e == cudaSuccess) *shape = strip_shape(P.nx, P.ny, nsm);
-  return e;
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((P.nx + F32_TX - 1) / F32_TX) * ((P.ny + F32_TY - 1) / F32_TY);
+  if (!learned || tiles >= (long long)LEARNED_STRIP_WAVES * HYDRO_F32_MINB * nsm) *shape = strip_shape(P.nx, P.ny, nsm);
+  return cudaSuccess;
 }
 
 template <int MODE>
@@ -223,7 +228,7 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
   const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 8;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
-  return launch_step_kernel(false, march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
+  return launch_step_kernel<float, MODE>(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
                             Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
@@ -235,13 +240,15 @@ cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout
                                  unsigned int* work) {
   static std::atomic<unsigned long long> attr_done{0};
   const size_t smem = TileLayout<float, F32_TX, F32_TY>::bytes;
-  cudaError_t e = smem_attr_once(learned_tiles_kernel<FUSED>, std::max(smem, STEP_SMEM_MAX), attr_done);
+  cudaError_t e = smem_attr_once(learned_tiles_kernel<FUSED>, smem, attr_done);
   int nsm = 0;
   if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
-  return launch_step_kernel(false, learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host,
-                            sc_dev, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp, work);
+  learned_tiles_kernel<FUSED><<<3 * nsm, 320, smem, stream>>>(P, Uin, Uout, sc_host, sc_dev, sc_next, scr, tmax,
+                                                             tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp,
+                                                             work);
+  return cudaGetLastError();
 }
 
 }  // namespace hydro

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
   constexpr int PQ = L::PQ, PC = L::PC, PF = L::PF, nQ = L::nQ, nC = L::nC, nF = L::nF;
   constexpr int kn = DIR == 0 ? 1 : 2, kt = DIR == 0 ? 2 : 1;  // normal / transverse momentum components
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  step_begin(Uin, sc_dev);
+  step_begin();
   R* sq = reinterpret_cast<R*>(smem_raw);  // [4][nQ] primitives, face frame
   R* sG = sq;                               // [4][nF] fluxes (conserved order), after stage 2
   R* sxi = sq + 4 * nQ;                     // [nC]
@@ -89,18 +89,14 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
 
   SP<R> s;
   s.load(P);
-  const StepScalars& sc = sc_dev ? *sc_dev : sc_host;
-  R sigma;
-  if constexpr (is_f32<R>())
-    sigma = DIR == 0 ? sc.sigx_f : sc.sigy_f;
+  StepFactors<R> f;
+  if (sc_dev)
+    f.load_ordered(sc_dev);
   else
-    sigma = DIR == 0 ? sc.sigx : sc.sigy;
+    f.load(sc_host);
+  const R sigma = DIR == 0 ? f.sigx : f.sigy;
   const R h = DIR == 0 ? s.dx : s.dy;
-  R hdtg;  // dt g / 2
-  if constexpr (is_f32<R>())
-    hdtg = sc.hdtg_f;
-  else
-    hdtg = sc.hdtg;
+  const R hdtg = f.hdtg;  // dt g / 2
   const int n = DIR == 0 ? P.nx : P.ny;      // interior cells along a line
   const int nlines = DIR == 0 ? P.ny : P.nx;
   const int bt = DIR == 0 ? blockIdx.x : blockIdx.y;  // tile along the sweep
@@ -124,7 +120,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
     if (a >= P.ng && a < P.ng + n) {
       const size_t o = interior_offset(a, l);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = __ldg(Uin + o + k * plane);
+      for (int k = 0; k < 4; ++k) v[k] = ld_ordered(Uin + o + k * plane);
     } else {
       bc_cell(P, Uin, DIR == 0 ? a : l, DIR == 0 ? l : a, plane, v);
     }
@@ -151,7 +147,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
         sweep_item<DIR, PQ, NL>(e, a, l);
         const size_t o = interior_offset(a0 - 4 + a, clamp_line(l0 + l));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) Ul[it][k] = __ldg(Uin + o + k * plane);
+        for (int k = 0; k < 4; ++k) Ul[it][k] = ld_ordered(Uin + o + k * plane);
       }
     }
 #pragma unroll
@@ -287,7 +283,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
     R Un[4], U0[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      U0[k] = __ldg(Uin + o + k * plane);
+      U0[k] = ld_ordered(Uin + o + k * plane);
       Un[k] = U0[k] + sigma * (sG[k * nF + g] - sG[k * nF + g + L::FA]);
     }
     if (DIR == 1 && P.use_grav) {
@@ -310,7 +306,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
   }
   flush_counters(cnt, scr);
   if constexpr (FUSED) {
-    finish_fused_step(P, cmin, &sc, sc_next, scr, tmax, 1u, gridDim.x * gridDim.y);
+    finish_fused_step(P, cmin, sc_dev, sc_next, scr, tmax, 1u, gridDim.x * gridDim.y);
   }
 }
 
@@ -332,12 +328,12 @@ struct Sweep {
     if (sc_next) {
       e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, std::max(L::bytes, STEP_SMEM_MAX), done_fused);
       if (e != cudaSuccess) return e;
-      return launch_step_kernel(!is_f32<R>(), sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+      return launch_step_kernel<R, MODE>(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
                                 sc_host, sc_dev, scr, check_state, sc_next, tmax);
     } else {
       e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, std::max(L::bytes, STEP_SMEM_MAX), done_plain);
       if (e != cudaSuccess) return e;
-      return launch_step_kernel(!is_f32<R>(), sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+      return launch_step_kernel<R, MODE>(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
                                 sc_host, sc_dev, scr, check_state, (StepScalars*)nullptr, 0.0);
     }
   }
