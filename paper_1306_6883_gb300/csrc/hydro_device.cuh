@@ -252,6 +252,11 @@ __device__ __forceinline__ float ld_ordered(const float* p) {
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
   return v;
 }
+__device__ __forceinline__ float2 ld_ordered2(const float* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
 __device__ __forceinline__ double ld_ordered(const double* p) {
   double v;
   asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));

@@ -17,9 +17,9 @@
 // and its last block advances the time and writes the next step's factors, as the fused unsplit step does.
 // Shared memory is laid out so that the load enumeration is also the storage order: along-the-line
 // positions are fastest for x sweeps (rows), lines are fastest for y sweeps (columns), so both load
-// consecutive x addresses with consecutive threads.  Instantiated for FP32 in k_split.cu and for FP64 in
-// k_split_f64.cu, which is compiled without multiply-add contraction (each expression then rounds like the
-// plain C implementation of the method).
+// consecutive x addresses with consecutive threads.  Instantiated for FP64 in k_split_f64.cu and
+// k_split_ppm_f64.cu, which are compiled without multiply-add contraction (each expression then rounds like the
+// plain C implementation of the method); the FP32 sweeps are those of sweep_march.cuh.
 #pragma once
 #include <atomic>
 
@@ -56,16 +56,8 @@ __device__ __forceinline__ void sweep_item(int e, int& a, int& l) {
   }
 }
 
-// Threads of the FP32 sweep CTAs (overridable at compile time for sweeps of the launch shape).  Measured per
-// split step, KH 1024^2 / Sedov 2048^2: 256 threads 77.9 / 225 us, 384 threads (36 warps per SM, 56
-// registers) 70.3 / 206 us, 512 threads (two CTAs per SM) 77.3 / 245 us.
-#ifndef HYDRO_SWEEP_F32_NT
-#define HYDRO_SWEEP_F32_NT 384
-#endif
-constexpr int SWEEP_F32_NT = HYDRO_SWEEP_F32_NT;
-
-// Resident CTAs per SM the register allocator must allow (shared memory admits three tiles of either
-// precision's shapes).
+// Resident CTAs per SM the register allocator must allow (shared memory admits three tiles of either direction's
+// shape).
 #ifndef HYDRO_SWEEP_MINB
 #define HYDRO_SWEEP_MINB 3
 #endif
@@ -253,12 +245,8 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
     G[3] = F[3];
     if (s.cvisc > (R)0 && valid) {
       R av;
-      if constexpr (is_f32<R>()) {
-        av = s.cvisc * M<R>::mx0(sun[cL] - sun[cR]);
-      } else {
-        const R div = soft_div(sun[cR] - sun[cL], h);
-        av = s.cvisc * M<R>::mx0(-div * h);
-      }
+      const R div = soft_div(sun[cR] - sun[cL], h);
+      av = s.cvisc * M<R>::mx0(-div * h);
       R UL[4], UR[4];
       load_cell(fa - 1, l0 + l, UL);
       load_cell(fa, l0 + l, UR);
@@ -273,7 +261,7 @@ __global__ void __launch_bounds__(NT, HYDRO_SWEEP_MINB) sweep_kernel(KParams P, 
 
   // ---- 4. conservative update of the tile's interior cells
   constexpr int nU = LN * NL;
-  R cmin = is_f32<R>() ? (R)FLT_MAX : (R)DBL_MAX;
+  R cmin = (R)DBL_MAX;
   for (int e = tid; e < nU; e += NT) {
     int u, l;
     sweep_item<DIR, LN, NL>(e, u, l);
