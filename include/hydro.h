@@ -347,8 +347,8 @@ void hydro_batch_destroy(hydro_batch* b);
 hydro_status hydro_batch_set_riemann_model(hydro_batch* b, const hydro_mlp* m);
 
 /* Tile-shape autotuner: for every size class time `reps` launches of each candidate tile shape on the
- * current states (without advancing them) and keep the fastest.  chosen_shapes (optional) receives one
- * shape id per class.  Synchronises.  Cached graphs are dropped. */
+ * current states (without advancing them) and keep the fastest, or one shape for all classes where that is
+ * faster for the whole ensemble.  chosen_shapes (optional) receives one shape id per class.  Synchronises.  Cached graphs are dropped. */
 hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes);
 
 /* Size classes (largest first) and the tile shape each uses. */

@@ -10,7 +10,7 @@
 
 #include <atomic>
 
-#include "ctu_tile.cuh"
+#include "ctu_march.cuh"
 #include "hydro_batch_internal.h"
 
 namespace hydro {
@@ -104,6 +104,24 @@ static __device__ __noinline__ void member_tile_done(const BatchMember& m, doubl
   scr->step_blocks_done = 0u;
 }
 
+// A block's counters into the batch's.
+__device__ __forceinline__ void flush_batch_counters(TileCounters cnt, DevScratch* agg) {
+  if (cnt.nonconv) cnt.flags |= STATUS_NONCONV;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    cnt.solves += __shfl_xor_sync(0xffffffffu, cnt.solves, off);
+    cnt.iters += __shfl_xor_sync(0xffffffffu, cnt.iters, off);
+    cnt.nonconv += __shfl_xor_sync(0xffffffffu, cnt.nonconv, off);
+    cnt.flags |= __shfl_xor_sync(0xffffffffu, cnt.flags, off);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&agg->stats[0], (unsigned long long)cnt.solves);
+    atomicAdd(&agg->stats[1], (unsigned long long)cnt.iters);
+    if (cnt.nonconv) atomicAdd(&agg->stats[2], (unsigned long long)cnt.nonconv);
+    if (cnt.flags) atomicOr(&agg->status, cnt.flags);
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------
 // Persistent fused CTU step over a tile list (member, tile x, tile y, the member's tile count), largest
 // members first: each CTA takes the next tile from an atomic queue until the list is exhausted.  A tile
@@ -153,20 +171,54 @@ __global__ void __launch_bounds__(NT, is_f32<R>() ? 3 : 2) batch_step_kernel(con
     }
     __syncthreads();  // the tile's last shared-memory reads finish before the next tile's loads
   }
-  if (cnt.nonconv) cnt.flags |= STATUS_NONCONV;
+  flush_batch_counters(cnt, agg);
+}
+
+// The same over a list of strips (ctu_march.cuh) of NV columns and NH rows: FP32, from the acoustic start.  An
+// ensemble's members are cut like its tiles, so a strip's item is a tile's.
+template <int NV, int NH, int NT>
+__global__ void __launch_bounds__(NT, MARCH_SM_THREADS / NT) batch_march_kernel(const BatchMember* __restrict__ mem,
+                                                       const int4* __restrict__ tiles, int ntiles,
+                                                       unsigned int* __restrict__ queue, int parity,
+                                                       DevScratch* __restrict__ agg, int advance) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ int cur;
+  __shared__ float wmin[NT / 32];
+  __shared__ KParams sP;
+  TileCounters cnt;
+  int member = -1;
+  while (true) {
+    if (threadIdx.x == 0) cur = (int)atomicAdd(queue, 1u);
+    __syncthreads();  // also: the strip's last shared-memory reads finish before the next one's writes
+    const int k = cur;
+    if (k >= ntiles) break;
+    const int4 t = tiles[k];
+    const BatchMember& m = mem[t.x];
+    if (t.x != member) {
+      for (int i = threadIdx.x; i < (int)(sizeof(KParams) / 4); i += NT)
+        reinterpret_cast<unsigned int*>(&sP)[i] = reinterpret_cast<const unsigned int*>(&m.P)[i];
+      member = t.x;
+      __syncthreads();
+    }
+    SP<float> s;
+    s.load(sP);
+    StepFactors<float> f;
+    f.load(m.scr->scf[parity]);
+    float cmin = FLT_MAX;
+    const int x0 = t.y * NV, y0 = t.z * NH;
+    ctu_march<FACE_PLAIN, true>(sP, s, f, (const float*)m.U[parity], (float*)m.U[1 - parity], sP.ng + x0,
+                                min(NV, sP.nx - x0), sP.ng + y0, min(NH, sP.ny - y0), smem_raw, cnt, nullptr, &cmin);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    cnt.solves += __shfl_xor_sync(0xffffffffu, cnt.solves, off);
-    cnt.iters += __shfl_xor_sync(0xffffffffu, cnt.iters, off);
-    cnt.nonconv += __shfl_xor_sync(0xffffffffu, cnt.nonconv, off);
-    cnt.flags |= __shfl_xor_sync(0xffffffffu, cnt.flags, off);
+    for (int off = 16; off > 0; off >>= 1) cmin = fminf(__shfl_xor_sync(0xffffffffu, cmin, off), cmin);
+    if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = cmin;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float b = wmin[0];
+      for (int w = 1; w < NT / 32; ++w) b = wmin[w] < b ? wmin[w] : b;
+      member_tile_done(m, (double)b, t.w, parity, advance);
+    }
   }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&agg->stats[0], (unsigned long long)cnt.solves);
-    atomicAdd(&agg->stats[1], (unsigned long long)cnt.iters);
-    if (cnt.nonconv) atomicAdd(&agg->stats[2], (unsigned long long)cnt.nonconv);
-    if (cnt.flags) atomicOr(&agg->status, cnt.flags);
-  }
+  flush_batch_counters(cnt, agg);
 }
 
 template <typename R, int TX, int TY, int NT, int MODE = FACE_PLAIN>
@@ -211,5 +263,47 @@ struct BatchStep {
 };
 template <typename R, int TX, int TY, int NT, int MODE>
 std::atomic<int> BatchStep<R, TX, TY, NT, MODE>::blocks_per_sm[64] = {};
+
+template <int NV, int NH, int NT>
+struct BatchMarch {
+  // per device (function attributes and occupancy belong to the device's context): set by prepare()
+  static std::atomic<int> blocks_per_sm[64];
+  static cudaError_t prepare() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64) return cudaErrorInvalidDevice;
+    if (blocks_per_sm[dev].load(std::memory_order_relaxed) > 0) return cudaSuccess;
+    const size_t smem = march_bytes(NT);
+    e = cudaFuncSetAttribute(batch_march_kernel<NV, NH, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+    if (e != cudaSuccess) return e;
+    int b = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, batch_march_kernel<NV, NH, NT>, NT, smem);
+    if (e != cudaSuccess) return e;
+    blocks_per_sm[dev].store(b > 0 ? b : 1, std::memory_order_relaxed);
+    return cudaSuccess;
+  }
+  static cudaError_t launch(const BatchMember* mem, const int4* tiles, int ntiles, unsigned int* queue, int parity,
+                            DevScratch* agg, cudaStream_t stream, int* grid_out, int advance) {
+    cudaError_t e = prepare();
+    if (e != cudaSuccess) return e;
+    int dev = 0, nsm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    int grid = nsm * blocks_per_sm[dev].load(std::memory_order_relaxed);
+    if (grid > ntiles) grid = ntiles;
+    if (grid_out) *grid_out = grid;
+    if (grid <= 0) return cudaSuccess;
+    e = cudaMemsetAsync(queue, 0, sizeof(unsigned int), stream);
+    if (e != cudaSuccess) return e;
+    batch_march_kernel<NV, NH, NT><<<grid, NT, march_bytes(NT), stream>>>(
+        mem, tiles, ntiles, queue, parity, agg, advance);
+    return cudaGetLastError();
+  }
+};
+template <int NV, int NH, int NT>
+std::atomic<int> BatchMarch<NV, NH, NT>::blocks_per_sm[64] = {};
 
 }  // namespace hydro

@@ -36,6 +36,8 @@ __device__ __forceinline__ void q_st(float4* a, int i, const float v[4]) {
   a[i] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// A strip's registers (128 a thread) let 512 threads share an SM: four strips of 128 columns.
+constexpr int MARCH_MAX_THREADS = 128, MARCH_SM_THREADS = 512;
 constexpr int MARCH_ROWS = 6;  // rows of primitives and of U^n a strip holds: c - 2 .. c + 3 around the traced row c
 
 // Shared memory of a strip of `threads` columns: the two row rings, five exchange rows of quadruples (MC slopes,

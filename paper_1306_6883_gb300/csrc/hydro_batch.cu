@@ -129,7 +129,7 @@ static cudaError_t build_tiles(hydro_batch* b, SizeClass& c, int shape) {
   c.ntiles = (int)tiles.size();
   c.shape = shape;
   // TMA descriptors of the class's members for this tile box (members without them load cell by cell)
-  if (e == cudaSuccess && b->d_tmaps) {
+  if (e == cudaSuccess && b->d_tmaps && shape < hydro::kNumLearnedShapes) {
     for (int m : c.members) {
       CUtensorMap maps[2];
       BatchMember& bm = b->hmem[m];
@@ -163,6 +163,24 @@ static cudaError_t enqueue_run(hydro_batch* b, int nsteps, int p0, cudaStream_t 
                             s, nullptr, b->d_tmaps, 1, batch_model(b));
     }
   return e;
+}
+
+// Time of one step of every group (milliseconds for reps of them after an untimed one; time does not advance).
+static float time_groups(hydro_batch* b, int reps, cudaEvent_t e0, cudaEvent_t e1, cudaError_t* err) {
+  cudaError_t e = cudaSuccess;
+  for (int r = 0; r <= reps && e == cudaSuccess; ++r) {
+    if (r == 1) cudaEventRecord(e0, b->stream);
+    for (auto& g : b->groups)
+      if (e == cudaSuccess)
+        e = hydro::batch_step(b->precision, g.shape, b->d_mem, g.d_tiles, g.ntiles, g.d_queue, b->parity, b->d_agg,
+                              b->stream, nullptr, b->d_tmaps, 0, batch_model(b));
+  }
+  cudaEventRecord(e1, b->stream);
+  if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+  float ms = 1e30f;
+  if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+  *err = e;
+  return ms;
 }
 
 extern "C" {
@@ -295,8 +313,7 @@ hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes) 
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  const int nshape = b->precision == HYDRO_FP64 ? 1 : hydro::kNumTileShapes;
-  int ci = 0;
+  const int nshape = b->precision == HYDRO_FP64 ? 1 : b->learned ? hydro::kNumLearnedShapes : hydro::kNumTileShapes;
   for (auto& c : b->classes) {
     float best = 1e30f;
     int best_shape = 0;
@@ -318,12 +335,31 @@ hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes) 
       }
     }
     if (e == cudaSuccess) e = build_tiles(b, c, best_shape);
-    if (chosen_shapes) chosen_shapes[ci] = best_shape;
-    ++ci;
+  }
+  if (e == cudaSuccess) e = rebuild_groups(b);
+  // The classes' own best shapes make a launch each and leave a tail each, so one shape for all may be faster yet (48
+  // members of 64^2 to 512^2: 331 us per step against 300 in strips of 88x32).
+  if (e == cudaSuccess && b->groups.size() > 1) {
+    std::vector<int> best_mix;
+    for (const auto& c : b->classes) best_mix.push_back(c.shape);
+    float best = time_groups(b, reps, e0, e1, &e);
+    for (int sh = 0; sh < nshape && e == cudaSuccess; ++sh) {
+      for (auto& c : b->classes)
+        if (e == cudaSuccess) e = build_tiles(b, c, sh);
+      if (e == cudaSuccess) e = rebuild_groups(b);
+      const float ms = e == cudaSuccess ? time_groups(b, reps, e0, e1, &e) : 1e30f;
+      if (e == cudaSuccess && ms < best) {
+        best = ms;
+        best_mix.assign(b->classes.size(), sh);
+      }
+    }
+    for (size_t k = 0; k < b->classes.size() && e == cudaSuccess; ++k) e = build_tiles(b, b->classes[k], best_mix[k]);
+    if (e == cudaSuccess) e = rebuild_groups(b);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (e == cudaSuccess) e = rebuild_groups(b);
+  if (chosen_shapes)
+    for (size_t k = 0; k < b->classes.size(); ++k) chosen_shapes[k] = b->classes[k].shape;
   // the trial launches counted solves; clear the aggregate counters
   if (e == cudaSuccess) e = hydro::init_scratch(b->d_agg, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);

@@ -23,6 +23,7 @@ struct TileShape {
 };
 extern const TileShape kTileShapes[];
 extern const int kNumTileShapes;
+extern const int kNumLearnedShapes;  // the first so many serve the learned start and load by TMA
 
 // tab[b] = (member, first cell, member's block count, 0); advance = 0 leaves time and step count alone; the
 // member's factors are also written to scf[parity] for the fused step

@@ -17,7 +17,11 @@ cudaError_t batch_dt(int precision, const BatchMember* mem, const int4* tab, int
 // Tile shapes the autotuner chooses from (index = shape id).
 const TileShape kTileShapes[] = {
     {32, 16, 384}, {16, 16, 256}, {32, 8, 256}, {32, 16, 256},
+    // strips (ctu_march.cuh), not with the learned start: 48 quadrant problems of 64^2 to 512^2 take 339 us per step in
+    // 32x16 tiles (the first shape), 307 in strips of 88x16, 334 of 120x16, 318 of 56x16, 300 of 88x32
+    {88, 16, 96}, {120, 16, 128}, {56, 16, 64}, {88, 32, 96},
 };
+const int kNumLearnedShapes = 4;
 const int kNumTileShapes = sizeof(kTileShapes) / sizeof(kTileShapes[0]);
 
 cudaError_t batch_step(int precision, int shape, const BatchMember* mem, const int4* tiles, int ntiles,
@@ -47,6 +51,10 @@ cudaError_t batch_step(int precision, int shape, const BatchMember* mem, const i
                                                               tmaps, advance);
     case 3: return BatchStep<float, 32, 16, 256>::launch(mem, tiles, ntiles, queue, parity, agg, stream, grid_out,
                                                               tmaps, advance);
+    case 4: return BatchMarch<88, 16, 96>::launch(mem, tiles, ntiles, queue, parity, agg, stream, grid_out, advance);
+    case 5: return BatchMarch<120, 16, 128>::launch(mem, tiles, ntiles, queue, parity, agg, stream, grid_out, advance);
+    case 6: return BatchMarch<56, 16, 64>::launch(mem, tiles, ntiles, queue, parity, agg, stream, grid_out, advance);
+    case 7: return BatchMarch<88, 32, 96>::launch(mem, tiles, ntiles, queue, parity, agg, stream, grid_out, advance);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -57,6 +65,10 @@ cudaError_t batch_prepare(int precision) {
   if (e == cudaSuccess) e = BatchStep<float, 16, 16, 256>::prepare();
   if (e == cudaSuccess) e = BatchStep<float, 32, 8, 256>::prepare();
   if (e == cudaSuccess) e = BatchStep<float, 32, 16, 256>::prepare();
+  if (e == cudaSuccess) e = BatchMarch<88, 16, 96>::prepare();
+  if (e == cudaSuccess) e = BatchMarch<120, 16, 128>::prepare();
+  if (e == cudaSuccess) e = BatchMarch<56, 16, 64>::prepare();
+  if (e == cudaSuccess) e = BatchMarch<88, 32, 96>::prepare();
   if (e == cudaSuccess) e = BatchStep<float, 32, 16, 384, FACE_LEARNED>::prepare();
   if (e == cudaSuccess) e = BatchStep<float, 16, 16, 256, FACE_LEARNED>::prepare();
   if (e == cudaSuccess) e = BatchStep<float, 32, 8, 256, FACE_LEARNED>::prepare();

@@ -6,8 +6,6 @@
 #include "ctu_march.cuh"
 
 namespace hydro {
-// A strip's registers (128 a thread) let 512 threads share an SM: four strips of 128 columns.
-constexpr int MARCH_MAX_THREADS = 128, MARCH_SM_THREADS = 512;
 
 // Work area of a learned step: the 32x16 tiles of the strips that met a strong face.  For each tile row, four words of
 // which a launch uses those of its first row (the list's length, the next tile to take, the blocks that are done, -);
