@@ -144,19 +144,33 @@ struct StripShape {
   int nv, nh, threads;
 };
 
-// The strips of an nx x ny grid on nsm SMs: the width (64, 96 or 128 threads, four columns of halo on each side) and
-// the number of rows that fill the SMs' strips evenly, in one wave where that takes at most 64 rows (in more, the SMs
-// even out strips of unlike cost: Sedov 4096^2 776 us per step in three or four waves, 860 in two, 1048 in one).  A row
-// takes a strip 3 to 4 us with one strip on the SM or with four, and each strip has six rows to load and two rows of
-// halo beside its own, so a step takes about 4 nh + 9 us a wave; a wave of three 32x16 tiles per SM is 16 us.  The
-// step takes the cheaper of the two, and tiles where the segments would be under five rows (their two halo rows are
-// then 40 % of the work, and the solves counted are twice a tile's).  Measured (us per step, tiles / strips): KH 64^2 16.8 / 15.1 (tiles),
-// 256^2 16.8 / 20.8 (tiles), 512^2 30.9 / 31.7 (tiles), 700x500 35.3 / 33.7, 1024^2 80.4 / 71.3, 1500x1300 139.8 / 116,
-// 2048^2 287 / 234, RT 317x951 39.6 / 36.2, Sedov 4096^2 1073 / 776.
-inline StripShape strip_shape(int nx, int ny, int nsm) {
+// What a step costs in us: strips waves * (row * nh + 9) + base - 9 (a row takes a strip `row` us with one strip on the SM
+// or with four; the rest is the rows loaded ahead, the launch and the tail), tiles 10 + tile * waves, where tiles share
+// the SMs evenly, so that waves are counted in fractions.  Tiles on reflecting or hydrostatic sides take 2.5 times as
+// long (bc_cell_clamped).
+struct StepCost {
+  double row, base, tile;
+};
+inline StepCost step_cost(const KParams& P) {
+  if (P.reconstruction == 1) return P.riemann_solver == 1 ? StepCost{4.0, 13.0, 17.0} : StepCost{5.1, 14.5, 19.0};
+  return P.riemann_solver == 1 ? StepCost{3.15, 12.0, 14.0} : StepCost{4.3, 14.0, 16.4};
+}
+
+// The strips of the grid on nsm SMs: the width (64, 96 or 128 threads, four columns of halo on each side) and the number
+// of rows that fill the SMs' strips evenly, in one wave where that takes at most 64 rows (in more, the SMs even out
+// strips of unlike cost: Sedov 4096^2 776 us per step in three or four waves, 860 in two, 1048 in one).  The step takes
+// the cheaper of strips and tiles, and tiles where the segments would be under five rows (their two halo rows are then
+// 40 % of the work, and the solves counted are twice a tile's).  Measured (us per step, tiles / strips):
+//   two-shock, PLM   512^2 29.0 / 34.4, 600x500 32.6 / 37.1, 700x500 33.7 / 35.0, RT 317x951 39.3 / 36.3, 800x640 43.8 /
+//                    46.4, 1000x800 65.9 / 65.7, KH 1024^2 79.4 / 78.0, 1300x1500 147 / 137, Sedov 2048^2 310 / 292
+//   HLLC             512^2 26.5 / 27.8, 700x500 30.9 / 28.3, 800x640 40.5 / 37.0, KH 1024^2 68.8 / 56.4
+//   two-shock, PPM   512^2 32.9 / 39.6, 800x640 50.6 / 53.7, 1000x700 69.8 / 75.9, KH 1024^2 92.3 / 90.5, 1300x1500 171 / 158
+inline StripShape strip_shape(const KParams& P, int nsm) {
   constexpr int MAX_ROWS = 64;
+  const StepCost k = step_cost(P);
+  const int nx = P.nx, ny = P.ny;
   StripShape best{0, 0, 0};
-  long long best_cost = 0;
+  double best_cost = 0.0;
   for (int threads = MARCH_MAX_THREADS; threads >= 64; threads -= 32) {
     const int n = (nx + threads - 9) / (threads - 8);  // strips across
     const long long slots = (long long)nsm * (MARCH_SM_THREADS / threads);
@@ -167,15 +181,16 @@ inline StripShape strip_shape(int nx, int ny, int nsm) {
       if (waves > (1 << 20)) break;
     }
     const int nh = (int)((ny + m - 1) / m);
-    const long long cost = waves * (4 * nh + 9);
+    const double cost = (double)waves * (k.row * nh + 9.0) + k.base - 9.0;
     if (best.nh == 0 || cost < best_cost) {
       best = StripShape{(nx + n - 1) / n, nh, threads};
       best_cost = cost;
     }
   }
-  const long long tiles = (long long)((nx + F32_TX - 1) / F32_TX) * ((ny + F32_TY - 1) / F32_TY);
-  const long long tile_waves = (tiles + HYDRO_F32_MINB * (long long)nsm - 1) / (HYDRO_F32_MINB * (long long)nsm);
-  if (best.nh < 5 || best_cost >= 16 * tile_waves) best.nh = 0;
+  const long long tx = (nx + F32_TX - 1) / F32_TX, ty = (ny + F32_TY - 1) / F32_TY;
+  const double tiles = (double)(tx * ty) + (P.bc_general ? 3.0 * (double)(tx + ty) : 0.0);
+  const double tile_cost = 10.0 + k.tile * tiles / (HYDRO_F32_MINB * (double)nsm);
+  if (best.nh < 5 || best_cost >= tile_cost) best.nh = 0;
   return best;
 }
 
@@ -192,7 +207,7 @@ inline cudaError_t choose_strips(const KParams& P, StripShape* shape, bool learn
   const cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((P.nx + F32_TX - 1) / F32_TX) * ((P.ny + F32_TY - 1) / F32_TY);
-  if (!learned || tiles >= (long long)LEARNED_STRIP_WAVES * HYDRO_F32_MINB * nsm) *shape = strip_shape(P.nx, P.ny, nsm);
+  if (!learned || tiles >= (long long)LEARNED_STRIP_WAVES * HYDRO_F32_MINB * nsm) *shape = strip_shape(P, nsm);
   return cudaSuccess;
 }
 

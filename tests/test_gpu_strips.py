@@ -19,9 +19,9 @@ def _problem(name, nx, ny):
     return {"kh": lambda: hp.kh(nx, ny, seed=1), "quad": lambda: hp.quad(nx, ny, seed=2)}[name]()
 
 
-# on 152 SMs the first four run in strips (of 128 and 64 threads, with ragged last strips and segments), the others in
-# tiles: too few rows to a segment, or fewer waves of tiles
-SIZES = [(1030, 700), (317, 951), (130, 2000), (100, 5000), (120, 130), (1500, 40), (1, 700)]
+# on 152 SMs the first three run in strips (ragged last strips and segments), the second and fourth with some of the
+# options or sides, the others in tiles: too few rows to a segment, or too few tiles
+SIZES = [(1030, 700), (317, 951), (100, 5000), (130, 2000), (700, 1100), (120, 130), (1500, 40), (1, 700)]
 
 
 @pytest.mark.parametrize("nx,ny", SIZES)
@@ -76,13 +76,14 @@ def test_strips_cut_into_bands_give_the_same_state(nx, ny):
     b.close()
 
 
+@pytest.mark.parametrize("nx,ny", [(1030, 700), (2100, 1800)])  # in tiles, in strips (sixteen waves of tiles)
 @pytest.mark.parametrize("gate", [None, (0.0, 0.0), (40.0, 1e9)])  # default, every face past it, none
-def test_learned_strips_hand_their_strong_faces_to_tiles(gate):
+def test_learned_strips_hand_their_strong_faces_to_tiles(gate, nx, ny):
     # an untrained network: its proposals change where the iterations start, not what they converge to
     import torch
     from paper_1306_6883_gb300 import hydro as H
     from paper_1306_6883_gb300.solver import Model, Solver, params_for
-    pr = hp.quad(1030, 700, seed=7)
+    pr = hp.quad(nx, ny, seed=7)
     po = oracle.params(pr.nx, pr.ny, bc=pr.bc)
     m = Model(seed=3)
     if gate:
