@@ -226,7 +226,8 @@ cudaError_t launch_march_step(const StripShape& sh, const KParams& P, const floa
 
 // band: tile rows of F32_TY cells (band.y <= 0: the whole step).  The segments of a band are short, since a band is a
 // fraction of the step and what counts is when its last row is done (KH 1024^2 chained host step, five bands: 188 us
-// with 4 rows, 194 with 8, 209 with 2; 4096^2: 2025 with 8, 2050 with 4).
+// with 4 rows, 194 with 8, 209 with 2; 8192^2 7.66 ms with 16 or 32, 7.72 with 8, and with the learned start 7.74 and
+// 8.13; 4096^2 2.00, 2.03 with 32).
 template <int MODE>
 cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, const float* Uin, float* Uout,
                                     const StepScalars* sc_cur, StepScalars* sc_next, DevScratch* scr, double tmax,
@@ -238,7 +239,7 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
   if (e != cudaSuccess) return e;
   const int row0 = band.y > 0 ? band.x * F32_TY : 0;
   const int rows = band.y > 0 ? min(band.y * F32_TY, P.ny - row0) : P.ny;
-  const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 8;
+  const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 16;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
   return launch_step_kernel<float, MODE>(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
