@@ -188,8 +188,8 @@ hydro_status hydro_advance(hydro_ctx* ctx, int nsteps, double tmax);
  * when tmax > 0).  The
  * first call after any other state change (hydro_step, hydro_step_device_dt, hydro_upload) computes this
  * step's dt with one extra reduction.  With split = 1: the two sweeps of hydro_step, the second one
- * reducing the next dt.  FP32 contexts with a learned model or a harvest run the separate passes instead.
- * Asynchronous. */
+ * reducing the next dt.  Contexts with a harvest run the separate passes instead.  Consecutive steps on a stream
+ * are launched ahead of one another's end (not while the stream is being captured).  Asynchronous. */
 hydro_status hydro_step_fused(hydro_ctx* ctx, double tmax);
 
 /* One step with host-resident state: host_in (pinned, layout of hydro_upload) is uploaded, stepped as
@@ -384,8 +384,8 @@ const char* hydro_build_info(void);
 
 /* 1 if the context's step kernels load tiles by TMA bulk tensor copies (FP32 contexts with ng a multiple of
  * 4 on a driver that provides the tensor-map encoder; tiles whose halo leaves the interior, or the padded
- * array for the unfused step, and the strips that larger grids run in are still loaded cell by cell), 0 otherwise or if ctx is NULL.  No paper
- * counterpart: how the data reaches shared memory does not change what a step computes. */
+ * array for the unfused step, the small tiles of small grids and the strips that larger grids run in are still
+ * loaded cell by cell), 0 otherwise or if ctx is NULL.  No paper counterpart: how the data reaches shared memory does not change what a step computes. */
 int hydro_tma_enabled(const hydro_ctx* ctx);
 
 /* Failure-path test of the bounded device-side wait (no paper counterpart).  drop = 1: the step runs in tiles
