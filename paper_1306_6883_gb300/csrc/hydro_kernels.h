@@ -88,7 +88,7 @@ cudaError_t ctu_step_fused_f64(const KParams& P, const double* Uin, double* Uout
 cudaError_t ctu_step_f64(const KParams& P, const double* Uin, double* Uout, const StepScalars& sc_host,
                          const StepScalars* sc_dev, DevScratch* scr, cudaStream_t stream);
 
-// One sweep of the dimensionally split variant (sweep_kernels.cuh) along dir (0: x, 1: y) of the state Uin
+// One sweep of the dimensionally split variant (FP32 sweep_march.cuh, FP64 sweep_kernels.cuh) along dir (0: x, 1: y) of the state Uin
 // into Uout (interior cells only; halo cells outside the domain are read through the boundary map, so Uin
 // needs no ghost fill), with sigma = dt/dx or dt/dy from sc_dev if not NULL, else sc_host.  check_state:
 // flag non-finite / non-positive cells of the result in the status word.  sc_next != NULL: the second sweep
