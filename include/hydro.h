@@ -189,7 +189,7 @@ hydro_status hydro_advance(hydro_ctx* ctx, int nsteps, double tmax);
  * first call after any other state change (hydro_step, hydro_step_device_dt, hydro_upload) computes this
  * step's dt with one extra reduction.  With split = 1: the two sweeps of hydro_step, the second one
  * reducing the next dt.  Contexts with a harvest run the separate passes instead.  Consecutive steps on a stream
- * are launched ahead of one another's end (not while the stream is being captured).  Asynchronous. */
+ * are launched ahead of one another's flush (not while the stream is being captured).  Asynchronous. */
 hydro_status hydro_step_fused(hydro_ctx* ctx, double tmax);
 
 /* One step with host-resident state: host_in (pinned, layout of hydro_upload) is uploaded, stepped as

@@ -185,17 +185,14 @@ cudaError_t launch_ctu_step(const KParams& P, const R* Uin, R* Uout, const StepS
 }
 
 // Fused steps follow one another on a stream, one launch each.  Their kernels are launched so that the next one's
-// blocks may be placed as soon as every block of this one has begun, and wait there for its end (step_begin, the
-// kernel's first statement): the launch itself then overlaps the step before (RT 317x951 39.0 -> 37.0 us per step, the
-// two sweeps of a split KH 1030x770 step 58.3 -> 53.9, HLLC KH 1024^2 60.4 -> 57.9).  What the
-// step before wrote is read with ld_ordered.
-__device__ __forceinline__ void step_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
-constexpr size_t SM_SMEM = 228 << 10, BLOCK_SMEM = 1 << 10;  // shared memory of an SM, and what a block takes beside its own
-constexpr size_t STEP_SMEM_MAX = SM_SMEM / 2 - BLOCK_SMEM + 128;  // the most launch_step_kernel asks for
+// blocks are placed as soon as every block of this one has exited, and wait there for what it wrote (step_begin, the
+// kernel's first statement): launch and flush then overlap (us per step: KH 64^2 FP32 11.0 -> 9.4, 384^2 21.1 -> 18.4,
+// split 512^2 27.3 -> 22.9, KH 64^2 FP64 77.0 -> 74.1).  Blocks placed any earlier hold SMs that another stream's
+// kernels could use, and unevenly, since SMs that are done first take more than their share.  Let in when this one's
+// blocks had begun, with shared memory padded to hold an SM to its even share, four KH 256^2 solvers on streams of
+// their own took 36.4 us per step (22.6 now, 24.7 without overlap); let in before the blocks' last reductions,
+// unpadded, FP64 192^2 alone took 154 (126 now).  What the step before wrote is read with ld_ordered.
+__device__ __forceinline__ void step_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 inline cudaError_t sm_count(int* nsm) {
   int dev = 0;
@@ -203,24 +200,14 @@ inline cudaError_t sm_count(int* nsm) {
   return e == cudaSuccess ? cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev) : e;
 }
 
-// Launches a fused step's kernel (its shared-memory limit raised to STEP_SMEM_MAX).  Blocks placed ahead of time go
-// where there is room, several to an SM that has none of the step before, so a grid of c blocks per SM or fewer asks for
-// as much shared memory as keeps an SM at c blocks (FP64 192^2, 144 tiles of which an SM takes two: 127 us per step
-// without the overlap, 199 with it, 124.5 with it and one tile to an SM; FP32 384^2 20.9, 22.5, 18.3).
-// Which steps overlap: in FP64 those of one block per SM or fewer, since a step with two tiles on some SMs loses more
-// than the launch (224x192 204.6 us without, 208 with; 64^2 75.3 and 73.2).  With the learned start, whose blocks differ
-// in cost, not those that fill some SMs' last places: SMs that are done early would take more than their share of the
-// next step (Sedov 400^2 38.6 us without, 40.2 with; 300^2 36.9 and 34.3).  Else all.
-template <typename R, int MODE, typename... Params, typename... Args>
+// Launches a fused step's kernel.
+template <typename... Params, typename... Args>
 cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
                                Args&&... args) {
   // a captured step keeps plain dependencies: graphs that a program edits or queries see the edges they always had
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  int nsm = 0;
-  cudaError_t e = cudaStreamIsCapturing(stream, &cap);
-  if (e == cudaSuccess) e = sm_count(&nsm);
+  const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
   if (e != cudaSuccess) return e;
-  const unsigned long long c = ((unsigned long long)grid.x * grid.y + nsm - 1) / nsm;
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -230,12 +217,7 @@ cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, int threads
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = &attr;
-  const bool overlap = !is_f32<R>() ? c == 1 : face_kind(MODE) != FACE_LEARNED || c != HYDRO_F32_MINB;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone && overlap ? 1 : 0;
-  if (cfg.numAttrs && c < 16) {
-    const size_t keep = (SM_SMEM / (c + 1) & ~(size_t)127) - BLOCK_SMEM + 128;  // c + 1 of these do not fit, c do
-    if (keep > smem) cfg.dynamicSmemBytes = keep;
-  }
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
@@ -292,14 +274,14 @@ cudaError_t launch_ctu_step_fused(const KParams& P, const R* Uin, R* Uout, const
                                   cudaStream_t stream, int2 band = make_int2(0, 0), const MlpBlob* mlp = nullptr) {
   const size_t smem = TileLayout<R, TX, TY>::bytes;
   static std::atomic<unsigned long long> attr_done{0};
-  cudaError_t e = smem_attr_once(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, std::max(smem, STEP_SMEM_MAX), attr_done);
+  cudaError_t e = smem_attr_once(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, smem, attr_done);
   if (e != cudaSuccess) return e;
   const int tx = (P.nx + TX - 1) / TX, ty = (P.ny + TY - 1) / TY;
   const int y0 = band.y > 0 ? band.x : 0, ny = band.y > 0 ? band.y : ty;
   if (y0 < 0 || ny <= 0 || y0 + ny > ty) return cudaErrorInvalidValue;
   dim3 grid(tx, ny);
-  return launch_step_kernel<R, MODE>(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin,
-                            Uout, sc_cur, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
+  return launch_step_kernel(ctu_step_fused_kernel<R, TX, TY, NT, MODE>, grid, NT, smem, stream, P, Uin, Uout,
+                            sc_cur, sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, y0,
                             (unsigned int)tx * (unsigned int)ty, mlp);
 }
 

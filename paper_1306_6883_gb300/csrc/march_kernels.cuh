@@ -236,16 +236,15 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
                                     cudaStream_t stream, int2 band, const MlpBlob* mlp = nullptr,
                                     unsigned int* work = nullptr) {
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e =
-      smem_attr_once(march_step_fused_kernel<MODE>, std::max(march_bytes(MARCH_MAX_THREADS), STEP_SMEM_MAX), attr_done);
+  const cudaError_t e = smem_attr_once(march_step_fused_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
   if (e != cudaSuccess) return e;
   const int row0 = band.y > 0 ? band.x * F32_TY : 0;
   const int rows = band.y > 0 ? min(band.y * F32_TY, P.ny - row0) : P.ny;
   const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 16;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
-  return launch_step_kernel<float, MODE>(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin,
-                            Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
+  return launch_step_kernel(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin, Uout,
+                            sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
 // A learned step of a grid that runs in strips: the strips, then the tiles they listed (three to an SM).

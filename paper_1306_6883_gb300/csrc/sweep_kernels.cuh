@@ -314,14 +314,14 @@ struct Sweep {
     const dim3 grid(DIR == 0 ? ta : tl, DIR == 0 ? tl : ta);
     cudaError_t e;
     if (sc_next) {
-      e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, std::max(L::bytes, STEP_SMEM_MAX), done_fused);
+      e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, L::bytes, done_fused);
       if (e != cudaSuccess) return e;
-      return launch_step_kernel<R, MODE>(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+      return launch_step_kernel(sweep_kernel<R, DIR, LN, NL, NT, true, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
                                 sc_host, sc_dev, scr, check_state, sc_next, tmax);
     } else {
-      e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, std::max(L::bytes, STEP_SMEM_MAX), done_plain);
+      e = smem_attr_once(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, L::bytes, done_plain);
       if (e != cudaSuccess) return e;
-      return launch_step_kernel<R, MODE>(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
+      return launch_step_kernel(sweep_kernel<R, DIR, LN, NL, NT, false, MODE>, grid, NT, L::bytes, stream, P, Uin, Uout,
                                 sc_host, sc_dev, scr, check_state, (StepScalars*)nullptr, 0.0);
     }
   }

@@ -371,20 +371,17 @@ template <int MODE>
 cudaError_t launch_sweep_f32(const KParams& P, const float* Uin, float* Uout, int dir, const StepScalars& sc_host,
                              const StepScalars* sc_dev, DevScratch* scr, int check_state, StepScalars* sc_next,
                              double tmax, cudaStream_t stream) {
-  static std::atomic<unsigned long long> done[4];
-  const int which = 2 * dir + (sc_next ? 1 : 0);
   int nsm = 0;
-  cudaError_t e = sm_count(&nsm);
+  const cudaError_t e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
   const auto kx = sc_next ? sweep_x_kernel<true, MODE> : sweep_x_kernel<false, MODE>;
   const auto ky = sc_next ? sweep_y_kernel<true, MODE> : sweep_y_kernel<false, MODE>;
-  if (e == cudaSuccess) e = dir == 0 ? smem_attr_once(kx, STEP_SMEM_MAX, done[which]) : smem_attr_once(ky, STEP_SMEM_MAX, done[which]);
-  if (e != cudaSuccess) return e;
   if (dir == 1) {
     int nh = sweep_share(P.ny, (long long)nsm * SWEEP_Y_BLOCKS * SWEEP_NT / P.nx, SWEEP_Y_ROWS);
     nh += nh & 1;
     const long long total = (long long)((P.ny + nh - 1) / nh) * P.nx;
-    return launch_step_kernel<float, MODE>(ky, dim3((unsigned int)((total + SWEEP_NT - 1) / SWEEP_NT)), SWEEP_NT, (size_t)0,
-                                           stream, P, Uin, Uout, sc_host, sc_dev, scr, check_state, sc_next, tmax, nh);
+    return launch_step_kernel(ky, dim3((unsigned int)((total + SWEEP_NT - 1) / SWEEP_NT)), SWEEP_NT, (size_t)0, stream, P,
+                              Uin, Uout, sc_host, sc_dev, scr, check_state, sc_next, tmax, nh);
   }
   int chunks = (P.nx + 55) / 56;
   int nv = (P.nx + chunks - 1) / chunks;
@@ -393,9 +390,9 @@ cudaError_t launch_sweep_f32(const KParams& P, const float* Uin, float* Uout, in
   const int rows = sweep_share(P.ny, (long long)nsm * SWEEP_X_BLOCKS * (SWEEP_NT / 32) / chunks, SWEEP_X_ROWS);
   const long long warps = (long long)chunks * ((P.ny + rows - 1) / rows);
   const int vec = P.ng % 2 == 0 && P.pitch % 2 == 0 && (size_t)Uin % 8 == 0 && (size_t)Uout % 8 == 0;
-  return launch_step_kernel<float, MODE>(kx, dim3((unsigned int)((warps + SWEEP_NT / 32 - 1) / (SWEEP_NT / 32))), SWEEP_NT,
-                                         (size_t)0, stream, P, Uin, Uout, sc_host, sc_dev, scr, check_state, sc_next, tmax,
-                                         nv, chunks, rows, vec);
+  return launch_step_kernel(kx, dim3((unsigned int)((warps + SWEEP_NT / 32 - 1) / (SWEEP_NT / 32))), SWEEP_NT, (size_t)0,
+                            stream, P, Uin, Uout, sc_host, sc_dev, scr, check_state, sc_next, tmax, nv, chunks, rows,
+                            vec);
 }
 
 }  // namespace hydro
