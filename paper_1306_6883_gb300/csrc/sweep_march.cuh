@@ -379,6 +379,10 @@ cudaError_t launch_sweep_f32(const KParams& P, const float* Uin, float* Uout, in
   if (dir == 1) {
     int nh = sweep_share(P.ny, (long long)nsm * SWEEP_Y_BLOCKS * SWEEP_NT / P.nx, SWEEP_Y_ROWS);
     nh += nh & 1;
+    // not shorter than eight rows while that leaves the SMs one and a half blocks each: what short segments repeat is
+    // time that other streams' kernels lose (KH 512^2, us per step alone / four at once: 4 rows 22.9 / 59.4, 8 rows 23.7 /
+    // 50.4; 384^2 2 and 4 rows 18.0 / 46.3 and 38.1, 6 rows 19.4 / 34.9)
+    while (nh < 8 && 2 * (long long)((P.ny + nh + 1) / (nh + 2)) * P.nx >= 3ll * nsm * SWEEP_NT) nh += 2;
     const long long total = (long long)((P.ny + nh - 1) / nh) * P.nx;
     return launch_step_kernel(ky, dim3((unsigned int)((total + SWEEP_NT - 1) / SWEEP_NT)), SWEEP_NT, (size_t)0, stream, P,
                               Uin, Uout, sc_host, sc_dev, scr, check_state, sc_next, tmax, nh);
