@@ -211,7 +211,7 @@ hydro_status hydro_step_host(hydro_ctx* ctx, const void* host_in, void* host_out
  * tmax and no other call that steps or replaces the state in between, this step's CFL time step is the
  * one the previous step reduced from the state it wrote (as hydro_step_fused keeps it), so no reduction
  * waits for the whole upload: each band of tile rows starts as soon as its rows and their 4-row halo
- * have arrived (five bands, eight above 2^21 cells), and the upload overlaps the step.  Otherwise the same as hydro_step_host.  The caller
+ * have arrived (eight bands, five in FP32 up to 2^21 cells), and the upload overlaps the step.  Otherwise the same as hydro_step_host.  The caller
  * must not modify host_out between the calls (the library checks the pointer, not the contents).  Same
  * results as hydro_step_host. */
 hydro_status hydro_step_host_chained(hydro_ctx* ctx, const void* host_in, void* host_out, double tmax);

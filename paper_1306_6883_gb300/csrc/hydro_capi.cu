@@ -720,13 +720,17 @@ static cudaError_t enqueue_host_step(hydro_ctx* c, const void* host_in, void* ho
   // bands of tile rows, in sixteenths: 1/8, 1/8, 1/4, 1/4, 1/4 when every band waits for the dt (small
   // first bands start the copies back early); when chained, eight bands of 1/16, 1/8, 1/8, 3/16, 3/16, 1/8,
   // 1/8, 1/16 (a small first band starts the copies back early, a small last one ends the step early after
-  // the whole upload), or up to 2^21 cells five bands of 3/16, 3/16, 1/4, 1/4, 1/8, since a band takes some 20 us
-  // however small it is (FP32, us per step with eight / five bands: KH 1024^2 194 / 188, 4096^2 2050 / 2156); grids
-  // of fewer than 16 tile rows split evenly into at most five bands
+  // the whole upload), or in FP32 up to 2^21 cells five bands of 3/16, 3/16, 1/4, 1/4, 1/8, since a band takes
+  // some 20 us in strips and 15 in tiles however small it is (us per step with eight / five bands: KH in tiles
+  // 256^2 61.1 / 56.0, 512^2 85.4 / 81.8, 700^2 124.7 / 119.4, PPM 1000x700 145.1 / 138.9; in strips 1024^2
+  // 184.3 / 179.2, 1448^2 332.0 / 323.3, 4096^2 2050 / 2156, HLLC 1024^2 178.6 / 179.4; learned 1024^2 177.7 /
+  // 181.8, 1448^2 324.0 / 319.7).  FP64 steps are bound by the step, to which a later first band and a larger last
+  // one only add (512^2 740.6 / 742.1, 1024^2 2793 / 2814, 1448^2 5607 / 5649).  Grids of fewer than 16 tile rows
+  // split evenly into at most five bands
   static const int sixteenths_dt[6] = {0, 2, 4, 8, 12, 16};
   static const int sixteenths_chain[NB + 1] = {0, 1, 3, 5, 8, 11, 13, 15, 16};
   static const int sixteenths_few[6] = {0, 3, 6, 10, 14, 16};
-  const bool few = (long long)ks.nx * ks.ny <= (1ll << 21);
+  const bool few = prec == HYDRO_FP32 && (long long)ks.nx * ks.ny <= (1ll << 21);
   const int ty = hydro::fused_tile_rows(prec, c->kp);
   const int tile_h = hydro::fused_tile_height(prec);  // cells per tile row
   const int nb = ty < 16 ? (ty < 5 ? ty : 5) : chained && !few ? NB : 5;
