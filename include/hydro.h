@@ -250,8 +250,11 @@ hydro_status hydro_conserved_totals_noalloc(const hydro_params* p, const void* d
  * HYDRO_ENONCONV, HYDRO_ETIMEOUT (a tile's TMA copy did not land within the bounded wait) recorded since
  * the last call.  After HYDRO_ETIMEOUT the state the steps wrote is not to be trusted: discard it and
  * upload a known state again (hydro_last_error says whether a copy was still outstanding when its tile
- * gave up, in which case later tiles on the same SM may have been overwritten as well).  Synchronises.  If stats is not NULL it receives
- * {riemann solves, riemann iterations, unconverged solves} accumulated since hydro_init. */
+ * gave up, in which case later tiles on the same SM may have been overwritten as well).  Synchronises.
+ * If stats is not NULL it receives {riemann solves, riemann iterations, unconverged solves} accumulated since
+ * hydro_init.  They count the work done, which depends on how a step is cut: a face that two tiles or two strips solve
+ * counts in each (the bands of host steps are strips of 4 or 16 rows), and so does what both launches of a learned
+ * step solve; the FP32 sweeps of a split step count every face once. */
 hydro_status hydro_sync_status(hydro_ctx* ctx, unsigned long long stats[3]);
 
 /* Copy a host array into / out of the current state.  host has the dense layout
@@ -272,7 +275,8 @@ hydro_status hydro_download(hydro_ctx* ctx, void* host);
  * steps (hydro_set_harvest).  FP32 contexts only.  Inference runs on the tensor cores (BF16 weights and
  * activations, FP32 accumulation), 32 faces per warp; a warp evaluates the network only when one of its
  * faces has |ln(p_L/p_R)|/2 > gate_dp or |u_L - u_R|/c_ref > gate_du, otherwise its faces start from the
- * acoustic estimate. */
+ * acoustic estimate.  Large grids step in strips from the acoustic estimate, and from the network only the 32x16
+ * tiles with a cell whose update reads a face past the gate that one iteration does not solve. */
 typedef struct hydro_mlp hydro_mlp;
 
 /* Create a network with He-normal weights drawn from `seed` (counter-based generator on the device).

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(NT, MARCH_SM_THREADS / NT) batch_march_kernel(
     float cmin = FLT_MAX;
     const int x0 = t.y * NV, y0 = t.z * NH;
     ctu_march<FACE_PLAIN, true>(sP, s, f, (const float*)m.U[parity], (float*)m.U[1 - parity], sP.ng + x0,
-                                min(NV, sP.nx - x0), sP.ng + y0, min(NH, sP.ny - y0), smem_raw, cnt, nullptr, &cmin);
+                                min(NV, sP.nx - x0), sP.ng + y0, min(NH, sP.ny - y0), smem_raw, cnt, &cmin);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) cmin = fminf(__shfl_xor_sync(0xffffffffu, cmin, off), cmin);
     if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = cmin;

@@ -23,6 +23,8 @@
 // depend on where a grid is cut into strips.
 #pragma once
 
+#include <float.h>
+
 #include "ctu_tile.cuh"
 
 namespace hydro {
@@ -42,9 +44,9 @@ constexpr int MARCH_ROWS = 6;  // rows of primitives and of U^n a strip holds: c
 
 // Shared memory of a strip of `threads` columns: the two row rings, five exchange rows of quadruples (MC slopes,
 // left states, hat fluxes, corrected left states, final fluxes) and six scalar rows (four of pressures, chi, the
-// y difference of v).
-__host__ __device__ constexpr size_t march_bytes(int threads) {
-  return sizeof(float) * (size_t)threads * (4 * (2 * MARCH_ROWS + 5) + 6);
+// y difference of v); a learned step's strip also four rows of notes (ctu_march).
+__host__ __device__ constexpr size_t march_bytes(int threads, bool learned = false) {
+  return sizeof(float) * (size_t)threads * (4 * (2 * MARCH_ROWS + 5) + (learned ? 10 : 6));
 }
 
 // energy of a ghost cell of a hydrostatic side (bc_cell) from its edge cell's values and its distance in cells
@@ -57,37 +59,91 @@ static __device__ __noinline__ float hydrostatic_energy(double gm1, double gdy, 
 }
 
 // Two face solves of a thread; the faces that count (n0, n1) add their iterations past the first to cnt.iters.
-template <int MODE>
+// slow: as for riemann_pair.
+template <int MODE, typename Slow>
 __device__ __forceinline__ void face_pair(const SP<float>& s, const float a[4], const float b[4], bool n0, float F[4],
-                                          const float c[4], const float d[4], bool n1, float G[4], TileCounters& cnt) {
+                                          const float c[4], const float d[4], bool n1, float G[4], TileCounters& cnt,
+                                          Slow&& slow) {
   if constexpr (face_kind(MODE) == FACE_HLLC) {
     hllc(s, a, b, F);
     hllc(s, c, d, G);
   } else {
-    riemann_pair(s, a, b, n0, F, c, d, n1, G, cnt.iters, cnt.nonconv);
+    riemann_pair(s, a, b, n0, F, c, d, n1, G, cnt.iters, cnt.nonconv, slow);
   }
 }
+template <int MODE>
+__device__ __forceinline__ void face_pair(const SP<float>& s, const float a[4], const float b[4], bool n0, float F[4],
+                                          const float c[4], const float d[4], bool n1, float G[4], TileCounters& cnt) {
+  face_pair<MODE>(s, a, b, n0, F, c, d, n1, G, cnt, [](bool&, bool&) {});
+}
 
-// Whether one of two counting faces is past the gate of the network mlp.
-__device__ __forceinline__ bool strong_pair(const MlpBlob* mlp, const float a[4], const float b[4], bool n0,
-                                            const float c[4], const float d[4], bool n1) {
-  const float ratio = __ldg(&mlp->gate_ratio), u4 = __ldg(&mlp->gate_u4);
-  return (n0 && strong_face(a, b, ratio, u4)) || (n1 && strong_face(c, d, ratio, u4));
+// Work area of a learned step (learned_work_bytes, all zero between steps).  For each row of 32x16 tiles, four words of
+// which a launch uses those of its first row (the list's length, the next tile to take, the blocks that are done, -);
+// the list of the tiles to be stepped with the network, a band's part beginning at its first tile; and for each tile
+// what its cells are in the strips: status flags with LISTED, and FLT_MAX's bits less those of their least CFL value.
+constexpr int LEARNED_TX = 32, LEARNED_TY = 16;
+struct LearnedWork {
+  static constexpr unsigned int LISTED = 0x80000000u;
+  unsigned int* counters;
+  int* list;
+  unsigned int *state, *slack;
+  int tx;
+  __device__ __forceinline__ LearnedWork(int nx, int ny, unsigned int* w, int by0) {
+    tx = (nx + LEARNED_TX - 1) / LEARNED_TX;
+    const int ty = (ny + LEARNED_TY - 1) / LEARNED_TY;
+    const size_t n = (size_t)tx * ty;
+    counters = w + 4 * (size_t)by0;
+    list = (int*)(w + 4 * (size_t)ty) + (size_t)by0 * tx;
+    state = w + 4 * (size_t)ty + n;
+    slack = state + n;
+  }
+  static constexpr size_t words(size_t tx, size_t ty) { return 4 * ty + 3 * tx * ty; }
+};
+
+// What a strip's warp hands in for the tile row ty (counted over the grid of nx by ny cells) of its cells: the lanes'
+// status flags and least CFL value to the tiles of the columns col they belong to (at most two tiles, from left to
+// right), and to the list, each once, the tiles of the columns x - 1, x and x + 1 where left, own and right say so.
+static __device__ __noinline__ void hand_in(int nx, int ny, unsigned int* work, int by0, int ty, int col, int x, bool left,
+                                            bool own, bool right, unsigned int flags, float cmin) {
+  const LearnedWork w(nx, ny, work, by0);
+  const int t = col / LEARNED_TX;
+  const size_t row = (size_t)ty * w.tx;
+  const int t0 = __shfl_sync(0xffffffffu, t, 0), t1 = __shfl_sync(0xffffffffu, t, 31);
+  const unsigned int slack = 0x7f7fffffu - __float_as_uint(cmin);
+  const unsigned int s0 = __reduce_max_sync(0xffffffffu, t == t0 ? slack : 0u);
+  const unsigned int s1 = __reduce_max_sync(0xffffffffu, t == t0 ? 0u : slack);
+  if ((threadIdx.x & 31) == 0) {
+    if (s0) atomicMax(&w.slack[row + t0], s0);
+    if (s1) atomicMax(&w.slack[row + t1], s1);
+  }
+  if (flags) atomicOr(&w.state[row + t], flags);
+  auto put = [&](int k) {
+    if (!(atomicOr(&w.state[row + k], LearnedWork::LISTED) & LearnedWork::LISTED))
+      w.list[atomicAdd(&w.counters[0], 1u)] = (int)row + k;
+  };
+  if (own) put(t);
+  if (left && !(own && (x - 1) / LEARNED_TX == t)) put((x - 1) / LEARNED_TX);
+  if (right && !(own && (x + 1) / LEARNED_TX == t)) put((x + 1) / LEARNED_TX);
 }
 
 // Steps the strip of nv columns (nv + 8 <= blockDim.x) and nh rows whose first interior cell is (i0, j0), padded
-// indices; smem holds march_bytes(blockDim.x).  MODE, FUSED, cfl_min as for ctu_tile.  FACE_LEARNED: the strip solves
-// from the acoustic start and gives up (returns true, its rows then partly written) after the row in which a face
-// is past the gate of mlp; its tiles are then to be stepped with the network.  Such faces are few and lie together, and
-// a network pass in a strip would hold up all its later rows (a blast's front kept strips for 1 ms).
+// indices; smem holds march_bytes(blockDim.x).  MODE, FUSED, cfl_min as for ctu_tile.
+//
+// FACE_LEARNED: the strip solves from the acoustic start.  The tiles that hold a cell whose update reads a strong face,
+// one past the gate of mlp whose first iteration makes no small step (one of the cell's own faces, or a hat face that
+// corrects their states), go on the list of work, to be stepped with the network by a second launch, which overwrites
+// them; so the strip leaves a strong face after that iteration.  Every strip that has a cell solves all those faces, so
+// the list does not depend on how the grid is cut.  The cells' status flags and CFL values go to the tiles' records
+// (hand_in), of which the second launch takes those of the tiles that were not listed.  The network itself in the strip
+// would hold up all its later rows (a blast's front kept strips for 1 ms).  Strong faces are noted per column and
+// iteration c, as bit c mod 32 of a word for each of the four solves, and handed in at the end of each tile row.
 template <int MODE, bool FUSED>
-__device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, const StepFactors<float>& f,
+__device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, const StepFactors<float>& f,
                                           const float* __restrict__ Uin, float* __restrict__ Uout, int i0, int nv, int j0,
-                                          int nh, unsigned char* smem, TileCounters& cnt, const MlpBlob* mlp,
-                                          float* cfl_min = nullptr) {
+                                          int nh, unsigned char* smem, TileCounters& cnt, float* cfl_min,
+                                          const MlpBlob* mlp = nullptr, unsigned int* work = nullptr, int by0 = 0) {
   static_assert(face_kind(MODE) != FACE_HARVEST, "the harvest steps in tiles");
   constexpr bool GATED = face_kind(MODE) == FACE_LEARNED;
-  bool strong = false;
   const int W = blockDim.x, x = threadIdx.x;  // column of the strip, its halo and copies of the last column past it
   const int xl1 = x > 0 ? x - 1 : 0, xr1 = x < W - 1 ? x + 1 : W - 1;
   float4* const ring_q = reinterpret_cast<float4*>(smem);
@@ -100,6 +156,7 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
   float* const ring_p = reinterpret_cast<float*>(x_flux + W);
   float* const x_chi = ring_p + 4 * W;
   float* const x_dv = x_chi + W;
+  uint2* const x_note = reinterpret_cast<uint2*>(x_dv + W);  // FACE_LEARNED: own column's only
 
   const int gi = i0 - 4 + (x < nv + 7 ? x : nv + 7);
   const int col = FUSED ? map_index(gi, P.ng, P.nx, P.bc[0], P.bc[1]) : (gi < P.NX ? gi : P.NX - 1);
@@ -190,6 +247,17 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
     slopes_x(j0 - 1, 3, a[2]);
     __syncthreads();
   }
+  // FACE_LEARNED: strong faces among the pair k of solves (0: hat faces along x and y, 1: final ones along y and x) of
+  // iteration c
+  auto strong = [&](int k, int c, bool sx, bool sy) {
+    if (sx || sy) {
+      uint2 v = x_note[k * W + x];
+      v.x |= sx ? 1u << (c & 31) : 0u;
+      v.y |= sy ? 1u << (c & 31) : 0u;
+      x_note[k * W + x] = v;
+    }
+  };
+  if constexpr (GATED) x_note[x] = x_note[W + x] = make_uint2(0, 0);
   int s3 = 0;  // ring slot of row c + 3
 #pragma unroll 1
   for (int c = j0 - 1; c <= j0 + nh; ++c) {
@@ -273,8 +341,17 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
     {
       float a[4], F[4];
       q_ld(x_l, xl1, a);
-      if constexpr (GATED) strong |= strong_pair(mlp, a, xr, on_xface, yl_c, yr, on_trace && c >= j0);
-      face_pair<MODE>(s, a, xr, on_xface, fxh, yl_c, yr, on_trace && c >= j0, F, cnt);
+      const bool on_y = on_trace && c >= j0;
+      face_pair<MODE>(s, a, xr, on_xface, fxh, yl_c, yr, on_y, F, cnt, [&](bool& ok0, bool& ok1) {
+        if constexpr (GATED) {
+          const float ratio = __ldg(&mlp->gate_ratio), u4 = __ldg(&mlp->gate_u4);
+          const bool sx = !ok0 & on_xface & strong_face(a, xr, ratio, u4);
+          const bool sy = !ok1 & on_y & strong_face(yl_c, yr, ratio, u4);
+          strong(0, c, sx, sy);
+          ok0 |= sx;
+          ok1 |= sy;
+        }
+      });
       q_st(x_hat, x, fxh);
       const float G[4] = {F[0], F[2], F[1], F[3]};
       float d[4];
@@ -303,8 +380,17 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
       ylc_new[0] = a[0]; ylc_new[1] = a[2]; ylc_new[2] = a[1]; ylc_new[3] = a[3];
       q_ld(x_lc, xl1, lc);
       float F[4];
-      if constexpr (GATED) strong |= strong_pair(mlp, ylc, yrc, on_cell && c >= j0, lc, xr_c, on_xface && c > j0);
-      face_pair<MODE>(s, ylc, yrc, on_cell && c >= j0, F, lc, xr_c, on_xface && c > j0, gx, cnt);
+      const bool on_y = on_cell && c >= j0, on_x = on_xface && c > j0;
+      face_pair<MODE>(s, ylc, yrc, on_y, F, lc, xr_c, on_x, gx, cnt, [&](bool& ok0, bool& ok1) {
+        if constexpr (GATED) {
+          const float ratio = __ldg(&mlp->gate_ratio), u4 = __ldg(&mlp->gate_u4);
+          const bool sy = !ok0 & on_y & strong_face(ylc, yrc, ratio, u4);
+          const bool sx = !ok1 & on_x & strong_face(lc, xr_c, ratio, u4);
+          strong(1, c, sy, sx);
+          ok0 |= sy;
+          ok1 |= sx;
+        }
+      });
       gy[0] = F[0]; gy[1] = F[2]; gy[2] = F[1]; gy[3] = F[3];
       q_ld(ring_u + sm * W, x, um);
       if (s.cvisc > 0.0f) {
@@ -330,11 +416,7 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
       ddu_c = ddu;
       ddv_c = ddv;
     }
-    if constexpr (GATED) {
-      if (__syncthreads_or(strong)) return true;
-    } else {
-      __syncthreads();
-    }
+    __syncthreads();
     // ---- update of row c - 1
     if (c > j0 && on_cell) {
       float fx1[4], Un[4];
@@ -365,13 +447,35 @@ __device__ __forceinline__ bool ctu_march(const KParams& P, const SP<float>& s, 
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) fy0[k] = gy[k];
+    if constexpr (GATED) {
+      if (c > j0 && ((c - P.ng) % LEARNED_TY == 0 || c == j0 + nh)) {  // row c - 1 ends a tile row or the strip
+        // its rows r0 .. c - 1 read the hat faces along x of iterations r0 - 1 to c and those along y of r0 to c, the final
+        // faces along y of r0 to c and along x of r0 + 1 to c; the next rows read those from c - 1 on again
+        const int n = (c - 1 - P.ng) % LEARNED_TY, r0 = c - 1 - n > j0 ? c - 1 - n : j0;
+        auto bits = [&](int from) {  // iterations from .. c
+          const unsigned int all = (2u << (c - from)) - 1u;
+          return __funnelshift_l(all, all, from & 31);
+        };
+        const uint2 h = x_note[x], g = x_note[W + x];
+        const unsigned int keep = 1u << (c & 31) | 1u << ((c - 1) & 31);
+        x_note[x] = make_uint2(h.x & keep, h.y & keep);
+        x_note[W + x] = make_uint2(g.x & keep, g.y & keep);
+        const bool hy = (h.y & bits(r0)) != 0, mine = (g.x & bits(r0)) != 0;
+        const bool both = ((h.x & bits(r0 - 1)) | (g.y & bits(r0 + 1))) != 0 || hy;
+        const int k = x < 4 ? 0 : x > nv + 3 ? nv - 1 : x - 4;  // the strip's column
+        hand_in(P.nx, P.ny, work, by0, (c - 1 - P.ng) / LEARNED_TY, i0 - P.ng + k, i0 - P.ng + x - 4,
+                both && x >= 5 && x <= nv + 4, (both || mine) && on_cell, hy && x >= 3 && x <= nv + 2, cnt.flags,
+                FUSED ? *cfl_min : FLT_MAX);
+        cnt.flags = 0;
+        if constexpr (FUSED) *cfl_min = FLT_MAX;
+      }
+    }
     s3 = s3 + 1 == MARCH_ROWS ? 0 : s3 + 1;
   }
   // every face above counted once; the iterations past the first were added as they ran
   const unsigned int solves = (on_xface ? 2 * nh + 2 : 0) + (on_trace ? nh + 1 : 0) + (on_cell ? nh + 1 : 0);
   cnt.solves += solves;
   if (face_kind(MODE) != FACE_HLLC) cnt.iters += solves;
-  return false;
 }
 
 }  // namespace hydro

@@ -1034,11 +1034,13 @@ __device__ __forceinline__ void riemann(const SP<float>& s, const float qL[4], c
 }
 
 // Two faces at once, so that their chains of dependent operations overlap: the fluxes of riemann(a, b) and
-// riemann(c, d) from the acoustic start.  more += the iterations past the first of the faces that count (n0, n1), nonconv += those that
-// did not converge.
+// riemann(c, d) from the acoustic start.  more += the iterations past the first of the faces that count (n0, n1),
+// nonconv += those that did not converge.  slow(ok0, ok1) is called where one step did not solve both, and may end the
+// iteration of one by setting it.
+template <typename Slow>
 __device__ __forceinline__ void riemann_pair(const SP<float>& s, const float a[4], const float b[4], bool n0, float F[4],
                                              const float c[4], const float d[4], bool n1, float G[4],
-                                             unsigned int& more, unsigned int& nonconv) {
+                                             unsigned int& more, unsigned int& nonconv, Slow&& slow) {
   TwoShockF r, q;
   r.start(s, a, b, 0.0f);
   q.start(s, c, d, 0.0f);
@@ -1046,6 +1048,7 @@ __device__ __forceinline__ void riemann_pair(const SP<float>& s, const float a[4
   q.step(s);
   bool ok0 = r.small_step(s), ok1 = q.small_step(s);
   if (!(ok0 && ok1)) {
+    slow(ok0, ok1);
     if (!ok0) {
       const int it = r.finish(s, 1, ok0);
       if (n0) { more += it - 1; nonconv += ok0 ? 0 : 1; }

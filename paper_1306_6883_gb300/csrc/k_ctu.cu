@@ -80,7 +80,7 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
 
 size_t learned_work_bytes(const KParams& P) {
   const size_t tx = (P.nx + F32_TX - 1) / F32_TX, ty = (P.ny + F32_TY - 1) / F32_TY;
-  return sizeof(unsigned int) * (4 * ty + 2 * tx * ty);
+  return sizeof(unsigned int) * LearnedWork::words(tx, ty);
 }
 
 }  // namespace hydro

@@ -7,35 +7,7 @@
 
 namespace hydro {
 
-// Work area of a learned step: the 32x16 tiles of the strips that met a strong face.  For each tile row, four words of
-// which a launch uses those of its first row (the list's length, the next tile to take, the blocks that are done, -);
-// then the list, a band's part beginning at its first tile; then a mark for each tile.  All zero between steps.
-struct LearnedWork {
-  unsigned int* counters;
-  int* list;
-  unsigned int* mark;
-  int tx;
-  __device__ __forceinline__ LearnedWork(const KParams& P, unsigned int* w, int by0) {
-    tx = (P.nx + F32_TX - 1) / F32_TX;
-    const int ty = (P.ny + F32_TY - 1) / F32_TY;
-    counters = w + 4 * by0;
-    list = (int*)(w + 4 * ty) + (size_t)by0 * tx;
-    mark = w + 4 * ty + (size_t)tx * ty;
-  }
-};
-
-// Puts the tiles that overlap a strip's cells [i0, i0 + nv) x [j0, j0 + nh) on the list, each once.
-__device__ __forceinline__ void list_strip(const KParams& P, unsigned int* work, int by0, int i0, int nv, int j0,
-                                           int nh) {
-  const LearnedWork w(P, work, by0);
-  const int bx0 = (i0 - P.ng) / F32_TX, bx1 = (i0 - P.ng + nv - 1) / F32_TX;
-  const int r0 = (j0 - P.ng) / F32_TY, r1 = (j0 - P.ng + nh - 1) / F32_TY;
-  const int n = (bx1 - bx0 + 1) * (r1 - r0 + 1);
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const int t = (r0 + k / (bx1 - bx0 + 1)) * w.tx + bx0 + k % (bx1 - bx0 + 1);
-    if (atomicExch(&w.mark[t], 1u) == 0u) w.list[atomicAdd(&w.counters[0], 1u)] = t;
-  }
-}
+static_assert(LEARNED_TX == F32_TX && LEARNED_TY == F32_TY, "the listed tiles are those of learned_tiles_kernel");
 
 template <int MODE>
 __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MAX_THREADS)
@@ -50,10 +22,7 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
   TileCounters cnt;
   const int i0 = P.ng + blockIdx.x * nv, j0 = P.ng + blockIdx.y * nh;
   const int cols = min(nv, P.ng + P.nx - i0), n = min(nh, P.ng + P.ny - j0);
-  if (ctu_march<MODE, false>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, mlp)) {
-    cnt = TileCounters();  // the strip's tiles count instead
-    list_strip(P, work, 0, i0, cols, j0, n);
-  }
+  ctu_march<MODE, false>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, nullptr, mlp, work);
   flush_counters(cnt, scr);
 }
 
@@ -86,21 +55,23 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
         cfl_value(s, u[0], u[1], u[2], u[3], cmin, cnt.flags);
       }
     }
-  } else if (ctu_march<MODE, true>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, mlp, &cmin)) {
-    cnt = TileCounters();  // the strip's tiles count instead
-    cmin = FLT_MAX;
-    list_strip(P, work, row0 / F32_TY, i0, cols, j0, n);
+  } else {
+    ctu_march<MODE, true>(P, s, f, Uin, Uout, i0, cols, j0, n, smem_raw, cnt, &cmin, mlp, work, row0 / LEARNED_TY);
   }
   flush_counters(cnt, scr);
   // a strip counts its rows, so that the bands of a step may cut it into segments of their own height; a learned step
   // is finished by the launch over the listed tiles
-  finish_fused_step<face_kind(MODE) != FACE_LEARNED>(P, cmin, sc_cur, sc_next, scr, tmax, (unsigned int)n, gridDim.x * (unsigned int)P.ny);
+  finish_fused_step<face_kind(MODE) != FACE_LEARNED>(P, cmin, sc_cur, sc_next, scr, tmax, (unsigned int)n,
+                                                     gridDim.x * (unsigned int)P.ny);
 }
 
-// The listed tiles of a learned step, from the network's proposals (blocks take them from the list until it is empty),
-// and for a fused step its end.  by0, rows: the tile rows of the launch (a band of the step, or all).  Bound by the chain
-// of stages of the few tiles it has.  Sedov 8192^2 learned, one step: 4.73 ms with all tiles in the tile kernel, 3.40 in
-// strips with this launch; with the network called from the strip's loop the strips on the blast's front took 1 ms each.
+// The second launch of a learned step: the listed tiles from the network's proposals (blocks take them from the list
+// until it is empty), which overwrite the strips' cells; the records of the tiles that were not listed; and for a fused
+// step its end.  by0, rows: the tile rows of the launch (a band of the step, or all).  Bound by the chain of stages of
+// the few tiles it has (11 us without any, 50 with those of a blast's front; ncu).  Sedov 8192^2 learned, one step: 4.73 ms
+// with all tiles in the tile kernel, 3.13 in strips with this launch (3.40 when a strip tested every face's gate and
+// gave up at the first strong one, and the list depended on the cut); with the network called from the strip's loop the
+// strips on the blast's front took 1 ms each.
 template <bool FUSED>
 __global__ void __launch_bounds__(320, 3)
     learned_tiles_kernel(KParams P, const float* __restrict__ Uin, float* __restrict__ Uout, StepScalars sc_host,
@@ -109,7 +80,8 @@ __global__ void __launch_bounds__(320, 3)
                          int by0, int rows, const MlpBlob* __restrict__ mlp, unsigned int* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int cur;
-  const LearnedWork w(P, work, by0);
+  step_begin();
+  const LearnedWork w(P.nx, P.ny, work, by0);
   TileCounters cnt;
   float cmin = FLT_MAX;
   const unsigned int n = *(volatile unsigned int*)&w.counters[0];
@@ -117,12 +89,14 @@ __global__ void __launch_bounds__(320, 3)
     SP<float> s;
     s.load(P);
     StepFactors<float> f;
-    f.load(sc_dev ? *sc_dev : sc_host);
+    if (sc_dev)
+      f.load_ordered(sc_dev);
+    else
+      f.load(sc_host);
     while (true) {
       if (threadIdx.x == 0) {
         const unsigned int k = atomicAdd(&w.counters[1], 1u);
         cur = k < n ? w.list[k] : -1;
-        if (cur >= 0) w.mark[cur] = 0u;
       }
       __syncthreads();
       const int t = cur;
@@ -132,6 +106,15 @@ __global__ void __launch_bounds__(320, 3)
                                                                       use_tma ? &tmap : nullptr);
       __syncthreads();  // the tile's last shared-memory reads finish before the next tile's loads
     }
+  }
+  const int first = by0 * w.tx, tiles = rows * w.tx;
+  for (int k = first + blockIdx.x * blockDim.x + threadIdx.x; k < first + tiles; k += gridDim.x * blockDim.x) {
+    const unsigned int state = w.state[k];
+    if (!(state & LearnedWork::LISTED)) {
+      cnt.flags |= state;
+      cmin = fminf(cmin, __uint_as_float(0x7f7fffffu - w.slack[k]));
+    }
+    w.state[k] = w.slack[k] = 0u;
   }
   flush_counters(cnt, scr);
   if constexpr (FUSED)
@@ -197,9 +180,9 @@ inline StripShape strip_shape(const KParams& P, int nsm) {
 }
 
 // The shape for a launch (nh == 0: tiles).  The withheld-copy test (hydro_test_drop_tile_copies) steps in tiles,
-// whose loads it is about.  A learned step's strips give up where they meet a strong face and cost a second launch, of
-// tiles three to an SM, so they need many waves of tiles to gain (us per step, tiles / strips, KH and quad problems:
-// 600x500 35.9 / 44.1 and 40.7 / 76.8, 1000^2 88 / 89 and 100 / 121, 1900^2 278 / 243 and 305 / 302).
+// whose loads it is about.  A learned step's strong faces cost a second launch, of tiles three to an SM, so its strips
+// need many waves of tiles to gain (us per step, tiles / strips, KH, quadrants and Sedov: 1000^2 84.5 / 73.6, 101 / 123
+// and 82.3 / 128; 1500x1300 148 / 123, 169 / 181 and 144 / 185; 1900^2 268 / 199, 292 / 274 and 256 / 282).
 constexpr int LEARNED_STRIP_WAVES = 16;
 
 inline cudaError_t choose_strips(const KParams& P, StripShape* shape, bool learned = false) {
@@ -217,11 +200,12 @@ template <int MODE>
 cudaError_t launch_march_step(const StripShape& sh, const KParams& P, const float* Uin, float* Uout,
                               const StepScalars& sc_host, const StepScalars* sc_dev, DevScratch* scr,
                               cudaStream_t stream, const MlpBlob* mlp = nullptr, unsigned int* work = nullptr) {
+  constexpr bool LEARNED = face_kind(MODE) == FACE_LEARNED;
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = smem_attr_once(march_step_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
+  const cudaError_t e = smem_attr_once(march_step_kernel<MODE>, march_bytes(MARCH_MAX_THREADS, LEARNED), attr_done);
   if (e != cudaSuccess) return e;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (P.ny + sh.nh - 1) / sh.nh);
-  march_step_kernel<MODE><<<grid, sh.threads, march_bytes(sh.threads), stream>>>(
+  march_step_kernel<MODE><<<grid, sh.threads, march_bytes(sh.threads, LEARNED), stream>>>(
       P, Uin, Uout, sc_host, sc_dev, scr, sh.nv, sh.nh, mlp, work);
   return cudaGetLastError();
 }
@@ -235,16 +219,17 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
                                     const StepScalars* sc_cur, StepScalars* sc_next, DevScratch* scr, double tmax,
                                     cudaStream_t stream, int2 band, const MlpBlob* mlp = nullptr,
                                     unsigned int* work = nullptr) {
+  constexpr bool LEARNED = face_kind(MODE) == FACE_LEARNED;
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = smem_attr_once(march_step_fused_kernel<MODE>, march_bytes(MARCH_MAX_THREADS), attr_done);
+  const cudaError_t e = smem_attr_once(march_step_fused_kernel<MODE>, march_bytes(MARCH_MAX_THREADS, LEARNED), attr_done);
   if (e != cudaSuccess) return e;
   const int row0 = band.y > 0 ? band.x * F32_TY : 0;
   const int rows = band.y > 0 ? min(band.y * F32_TY, P.ny - row0) : P.ny;
   const int nh = band.y <= 0 ? sh.nh : sh.nh < 32 ? 4 : 16;
   if (row0 < 0 || rows <= 0 || row0 + rows > P.ny) return cudaErrorInvalidValue;
   const dim3 grid((P.nx + sh.nv - 1) / sh.nv, (rows + nh - 1) / nh);
-  return launch_step_kernel(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads), stream, P, Uin, Uout,
-                            sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
+  return launch_step_kernel(march_step_fused_kernel<MODE>, grid, sh.threads, march_bytes(sh.threads, LEARNED), stream, P,
+                            Uin, Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
 // A learned step of a grid that runs in strips: the strips, then the tiles they listed (three to an SM).
@@ -260,10 +245,8 @@ cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout
   if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
-  learned_tiles_kernel<FUSED><<<3 * nsm, 320, smem, stream>>>(P, Uin, Uout, sc_host, sc_dev, sc_next, scr, tmax,
-                                                             tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp,
-                                                             work);
-  return cudaGetLastError();
+  return launch_step_kernel(learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host, sc_dev,
+                            sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp, work);
 }
 
 }  // namespace hydro
