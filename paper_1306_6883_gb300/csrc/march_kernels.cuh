@@ -72,8 +72,10 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
 // with all tiles in the tile kernel, 3.13 in strips with this launch (3.40 when a strip tested every face's gate and
 // gave up at the first strong one, and the list depended on the cut); with the network called from the strip's loop the
 // strips on the blast's front took 1 ms each.
+// Two blocks an SM: with three the registers (64) spilled 136 bytes in the chain (Sedov 3000^2 503 us per step, 488 with
+// two; 2200x2100 298 and 282).
 template <bool FUSED>
-__global__ void __launch_bounds__(320, 3)
+__global__ void __launch_bounds__(320, 2)
     learned_tiles_kernel(KParams P, const float* __restrict__ Uin, float* __restrict__ Uout, StepScalars sc_host,
                          const StepScalars* __restrict__ sc_dev, StepScalars* __restrict__ sc_next,
                          DevScratch* __restrict__ scr, double tmax, const __grid_constant__ CUtensorMap tmap, int use_tma,
@@ -180,9 +182,10 @@ inline StripShape strip_shape(const KParams& P, int nsm) {
 }
 
 // The shape for a launch (nh == 0: tiles).  The withheld-copy test (hydro_test_drop_tile_copies) steps in tiles,
-// whose loads it is about.  A learned step's strong faces cost a second launch, of tiles three to an SM, so its strips
-// need many waves of tiles to gain (us per step, tiles / strips, KH, quadrants and Sedov: 1000^2 84.5 / 73.6, 101 / 123
-// and 82.3 / 128; 1500x1300 148 / 123, 169 / 181 and 144 / 185; 1900^2 268 / 199, 292 / 274 and 256 / 282).
+// whose loads it is about.  A learned step's strong faces cost a second launch, so its strips need many waves of tiles
+// to gain (us per step, tiles / strips, KH, quadrants and Sedov: 1000^2 84.5 / 73.6, 101 / 123 and 82.3 / 128; 1500x1300
+// 148 / 123, 169 / 181 and 144 / 185; 1900^2 268 / 199, 292 / 274 and 256 / 282, with three blocks of the second launch
+// an SM).
 constexpr int LEARNED_STRIP_WAVES = 16;
 
 inline cudaError_t choose_strips(const KParams& P, StripShape* shape, bool learned = false) {
@@ -232,7 +235,7 @@ cudaError_t launch_march_step_fused(const StripShape& sh, const KParams& P, cons
                             Uin, Uout, sc_cur, sc_next, scr, tmax, row0, rows, sh.nv, nh, mlp, work);
 }
 
-// A learned step of a grid that runs in strips: the strips, then the tiles they listed (three to an SM).
+// A learned step of a grid that runs in strips: the strips, then the tiles they listed (two to an SM).
 template <bool FUSED>
 cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout, const StepScalars& sc_host,
                                  const StepScalars* sc_dev, StepScalars* sc_next, DevScratch* scr, double tmax,
@@ -245,7 +248,7 @@ cudaError_t launch_learned_tiles(const KParams& P, const float* Uin, float* Uout
   if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const int ty = (P.ny + F32_TY - 1) / F32_TY, by0 = band.y > 0 ? band.x : 0, rows = band.y > 0 ? band.y : ty;
-  return launch_step_kernel(learned_tiles_kernel<FUSED>, dim3(3 * nsm), 320, smem, stream, P, Uin, Uout, sc_host, sc_dev,
+  return launch_step_kernel(learned_tiles_kernel<FUSED>, dim3(2 * nsm), 320, smem, stream, P, Uin, Uout, sc_host, sc_dev,
                             sc_next, scr, tmax, tmap ? *tmap : CUtensorMap{}, tmap ? 1 : 0, by0, rows, mlp, work);
 }
 
