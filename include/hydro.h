@@ -350,10 +350,18 @@ void hydro_batch_destroy(hydro_batch* b);
  * where their gate opens.  m must outlive its use.  Captured graphs are dropped when m changes. */
 hydro_status hydro_batch_set_riemann_model(hydro_batch* b, const hydro_mlp* m);
 
-/* Tile-shape autotuner: for every size class time `reps` launches of each candidate tile shape on the
- * current states (without advancing them) and keep the fastest, or one shape for all classes where that is
- * faster for the whole ensemble.  chosen_shapes (optional) receives one shape id per class.  Synchronises.  Cached graphs are dropped. */
+/* Tile-shape autotuner: for every size class time `reps` launches of each candidate tile shape (ids 0 to 3 tiles, 4 to
+ * 7 strips, which the learned start has none of) on the current states (without advancing them) and keep the fastest,
+ * or one shape for all classes where that is faster for the whole ensemble.  It takes reps + 1 steps of the ensemble
+ * for each shape and as many for each shape as the only one.  chosen_shapes (optional) receives one shape id per
+ * class.  Synchronises.  Cached graphs are dropped.  FP32 results in different shapes agree to rounding, not bit for bit, and
+ * which shape is the fastest can depend on the run; hydro_batch_set_shape fixes it. */
 hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes);
+
+/* Step every member in tiles or strips of this shape (an id of hydro_batch_autotune; FP64 has shape 0 alone).  The
+ * default is shape 0.  Synchronises.  Cached graphs are dropped.  Returns HYDRO_EINVAL for an id that the members'
+ * precision or start does not have. */
+hydro_status hydro_batch_set_shape(hydro_batch* b, int shape);
 
 /* Size classes (largest first) and the tile shape each uses. */
 int hydro_batch_num_classes(const hydro_batch* b);

@@ -165,6 +165,10 @@ static cudaError_t enqueue_run(hydro_batch* b, int nsteps, int p0, cudaStream_t 
   return e;
 }
 
+static int num_shapes(const hydro_batch* b) {
+  return b->precision == HYDRO_FP64 ? 1 : b->learned ? hydro::kNumLearnedShapes : hydro::kNumTileShapes;
+}
+
 // Time of one step of every group (milliseconds for reps of them after an untimed one; time does not advance).
 static float time_groups(hydro_batch* b, int reps, cudaEvent_t e0, cudaEvent_t e1, cudaError_t* err) {
   cudaError_t e = cudaSuccess;
@@ -313,7 +317,7 @@ hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes) 
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  const int nshape = b->precision == HYDRO_FP64 ? 1 : b->learned ? hydro::kNumLearnedShapes : hydro::kNumTileShapes;
+  const int nshape = num_shapes(b);
   for (auto& c : b->classes) {
     float best = 1e30f;
     int best_shape = 0;
@@ -365,6 +369,16 @@ hydro_status hydro_batch_autotune(hydro_batch* b, int reps, int* chosen_shapes) 
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   drop_graphs(b);
   return e == cudaSuccess ? HYDRO_OK : fail(b, e, "autotune");
+}
+
+hydro_status hydro_batch_set_shape(hydro_batch* b, int shape) {
+  if (!b || shape < 0 || shape >= num_shapes(b)) return HYDRO_EINVAL;
+  cudaError_t e = cudaStreamSynchronize(b->stream);  // steps in flight read the tile lists
+  for (auto& c : b->classes)
+    if (e == cudaSuccess) e = build_tiles(b, c, shape);
+  if (e == cudaSuccess) e = rebuild_groups(b);
+  drop_graphs(b);
+  return e == cudaSuccess ? HYDRO_OK : fail(b, e, "set shape");
 }
 
 int hydro_batch_num_classes(const hydro_batch* b) { return b ? (int)b->classes.size() : 0; }

@@ -93,6 +93,7 @@ SIGNATURES = {
     "hydro_batch_destroy": (None, [_VP]),
     "hydro_batch_set_riemann_model": (ctypes.c_int, [_VP, _VP]),
     "hydro_batch_autotune": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
+    "hydro_batch_set_shape": (ctypes.c_int, [_VP, ctypes.c_int]),
     "hydro_batch_num_classes": (ctypes.c_int, [_VP]),
     "hydro_batch_class_info": (ctypes.c_int, [_VP, ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)] * 6),
     "hydro_batch_run": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int]),
@@ -288,6 +289,10 @@ def hydro_batch_autotune(b, reps=3):
     out = (ctypes.c_int * max(n, 1))()
     _bcheck(load().hydro_batch_autotune(b, int(reps), out), b, "hydro_batch_autotune")
     return list(out)[:n]
+
+
+def hydro_batch_set_shape(b, shape):
+    _bcheck(load().hydro_batch_set_shape(b, int(shape)), b, "hydro_batch_set_shape")
 
 
 def hydro_batch_classes(b):

@@ -156,6 +156,10 @@ class Ensemble:
     def autotune(self, reps=3):
         return H.hydro_batch_autotune(self.b, reps)
 
+    def set_shape(self, shape):
+        """Step every member in tiles or strips of one shape (an id that autotune may return)."""
+        H.hydro_batch_set_shape(self.b, shape)
+
     def set_model(self, model):
         """Start every member's Riemann iterations from `model` (a Model; the members need
         use_learned_guess = 1), or from the acoustic estimate again with None."""
