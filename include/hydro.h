@@ -394,6 +394,12 @@ const char* hydro_last_error(const hydro_ctx* ctx);
 /* Library build string (compute capability and options), never NULL. */
 const char* hydro_build_info(void);
 
+/* How hydro_step, hydro_step_device_dt and hydro_step_fused cut the context's grid on the current device: into strips
+ * (1) or tiles (0) of so many columns and rows, whichever the library's rule takes for the grid, the form of the step
+ * and the number of SMs (bands of host steps have rows of their own).  Each pointer may be NULL.  Returns HYDRO_EINVAL
+ * for a NULL or split context.  No paper counterpart: tests ask which kernel they reach. */
+hydro_status hydro_step_cut(const hydro_ctx* ctx, int* strips, int* columns, int* rows);
+
 /* 1 if the context's step kernels load tiles by TMA bulk tensor copies (FP32 contexts with ng a multiple of
  * 4 on a driver that provides the tensor-map encoder; tiles whose halo leaves the interior, or the padded
  * array for the unfused step, the small tiles of small grids and the strips that larger grids run in are still

@@ -889,6 +889,16 @@ const char* hydro_build_info(void) {
          "fp32 32x16/384 with TMA tile loads), march_step and march_step_fused (fp32 strips), batch fill/dt/step, totals, mlp";
 }
 
+hydro_status hydro_step_cut(const hydro_ctx* c, int* strips, int* columns, int* rows) {
+  if (!c || c->p.split) return HYDRO_EINVAL;
+  int cut[3];
+  if (hydro::step_cut(c->p.precision, c->kp, c->p.use_learned_guess == 1, cut) != cudaSuccess) return HYDRO_ECUDA;
+  if (strips) *strips = cut[0];
+  if (columns) *columns = cut[1];
+  if (rows) *rows = cut[2];
+  return HYDRO_OK;
+}
+
 int hydro_tma_enabled(const hydro_ctx* c) { return c ? c->tma_ok : 0; }
 
 hydro_status hydro_test_drop_tile_copies(hydro_ctx* c, int drop, unsigned int polls) {

@@ -36,6 +36,8 @@ cudaError_t ctu_step_fused(int precision, const KParams& P, const void* Uin, voi
                            cudaStream_t stream, int2 band = make_int2(0, 0), const MlpBlob* mlp = nullptr,
                            unsigned int* learned_work = nullptr);
 size_t learned_work_bytes(const KParams& P);
+// How a whole step is cut: strips (cut[0] = 1) or tiles of cut[1] columns and cut[2] rows.
+cudaError_t step_cut(int precision, const KParams& P, bool learned, int cut[3]);
 int fused_tile_rows(int precision, const KParams& P);
 int fused_tile_height(int precision);
 

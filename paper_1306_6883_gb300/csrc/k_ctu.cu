@@ -78,6 +78,17 @@ cudaError_t ctu_step(int precision, const KParams& P, const void* Uin, void* Uou
   }
 }
 
+cudaError_t step_cut(int precision, const KParams& P, bool learned, int cut[3]) {
+  StripShape sh{0, 0, 0};
+  bool small = false;
+  cudaError_t e = precision == 0 ? f64_small_tile(P, &small) : choose_strips(P, &sh, learned);
+  if (e == cudaSuccess && precision != 0 && !sh.nh) e = f32_small_tile(P, &small);
+  cut[0] = sh.nh > 0;
+  cut[1] = sh.nh ? sh.nv : precision == 0 ? F64_TX : small ? F32_SMALL_TX : F32_TX;
+  cut[2] = sh.nh ? sh.nh : precision == 0 ? (small ? F64_TY_SMALL : F64_TY) : small ? F32_SMALL_TY : F32_TY;
+  return e;
+}
+
 size_t learned_work_bytes(const KParams& P) {
   const size_t tx = (P.nx + F32_TX - 1) / F32_TX, ty = (P.ny + F32_TY - 1) / F32_TY;
   return sizeof(unsigned int) * LearnedWork::words(tx, ty);

@@ -105,6 +105,7 @@ SIGNATURES = {
     "hydro_batch_last_error": (ctypes.c_char_p, [_VP]),
     "hydro_last_error": (ctypes.c_char_p, [_VP]),
     "hydro_build_info": (ctypes.c_char_p, []),
+    "hydro_step_cut": (ctypes.c_int, [_VP] + [ctypes.POINTER(ctypes.c_int)] * 3),
     "hydro_tma_enabled": (ctypes.c_int, [_VP]),
     "hydro_test_drop_tile_copies": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint]),
 }
@@ -249,6 +250,13 @@ def hydro_step_host_chained(ctx, host_in_ptr, host_out_ptr, tmax=0.0):
 
 def hydro_build_info():
     return load().hydro_build_info().decode()
+
+
+def hydro_step_cut(ctx):
+    """("strips" or "tiles", columns, rows)"""
+    v = [ctypes.c_int() for _ in range(3)]
+    _check(load().hydro_step_cut(ctx, *[ctypes.byref(x) for x in v]), ctx, "hydro_step_cut")
+    return ("strips" if v[0].value else "tiles", v[1].value, v[2].value)
 
 
 def hydro_tma_enabled(ctx):
