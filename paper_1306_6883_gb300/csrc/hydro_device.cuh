@@ -472,54 +472,39 @@ __device__ __forceinline__ float2 slope_pair(int limiter, float2 qm2, float2 qm1
   return f2(pr.x > 0.f ? copysignf(mx, d4.x) : 0.f, pr.y > 0.f ? copysignf(my, d4.y) : 0.f);
 }
 
-// The limiter of four components at once from their one-sided differences dl = q0 - qm, dr = qp - q0 and
+// The FP32 limiter of four components at once from their one-sided differences dl = q0 - qm, dr = qp - q0 and
 // dd = qp - qm: the MC slopes (mc4), and the fourth-order slopes times xi from them and the neighbours' MC slopes
 // (slope4), with the operations and order of mc2, slope and slope_pair.
-template <typename R>
-__device__ __forceinline__ void mc4(const R dl[4], const R dr[4], const R dd[4], R m[4]) {
-  if constexpr (is_f32<R>()) {
+__device__ __forceinline__ void mc4(const float dl[4], const float dr[4], const float dd[4], float m[4]) {
 #pragma unroll
-    for (int h = 0; h < 4; h += 2) {
-      const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
-      const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
-      const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
-      const float mx = fminf(fabsf(dc.x), dlim.x), my = fminf(fabsf(dc.y), dlim.y);
-      m[h] = pr.x > 0.f ? copysignf(mx, dc.x) : 0.f;
-      m[h + 1] = pr.y > 0.f ? copysignf(my, dc.y) : 0.f;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) m[k] = limited64(dl[k], dr[k], sf_half(dd[k]));
+  for (int h = 0; h < 4; h += 2) {
+    const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
+    const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
+    const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
+    const float mx = fminf(fabsf(dc.x), dlim.x), my = fminf(fabsf(dc.y), dlim.y);
+    m[h] = pr.x > 0.f ? copysignf(mx, dc.x) : 0.f;
+    m[h + 1] = pr.y > 0.f ? copysignf(my, dc.y) : 0.f;
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void slope4(int limiter, R xi, const R dl[4], const R dr[4], const R dd[4], const R mL[4],
-                                       const R m0[4], const R mR[4], R dq[4]) {
+__device__ __forceinline__ void slope4(int limiter, float xi, const float dl[4], const float dr[4], const float dd[4],
+                                       const float mL[4], const float m0[4], const float mR[4], float dq[4]) {
   if (limiter != 2) {  // uniform over the launch: piecewise constant (0) or MC (1)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dq[k] = limiter == 0 ? (R)0 : xi * m0[k];
+    for (int k = 0; k < 4; ++k) dq[k] = limiter == 0 ? 0.0f : xi * m0[k];
     return;
   }
-  if constexpr (is_f32<R>()) {
 #pragma unroll
-    for (int h = 0; h < 4; h += 2) {
-      const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
-      const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
-      const float2 m = add2(f2(mR[h], mR[h + 1]), f2(mL[h], mL[h + 1]));
-      const float2 d4 = fma2(f2(4.0f / 3.0f), dc, mul2(f2(-1.0f / 6.0f), m));
-      const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
-      const float mx = fminf(fabsf(d4.x), dlim.x), my = fminf(fabsf(d4.y), dlim.y);
-      const float2 d = mul2(f2(xi), f2(pr.x > 0.f ? copysignf(mx, d4.x) : 0.f, pr.y > 0.f ? copysignf(my, d4.y) : 0.f));
-      dq[h] = d.x;
-      dq[h + 1] = d.y;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double d4 = (4.0 / 3.0) * sf_half(dd[k]) - (1.0 / 6.0) * (mR[k] + mL[k]);
-      dq[k] = xi * limited64(dl[k], dr[k], d4);
-    }
+  for (int h = 0; h < 4; h += 2) {
+    const float2 dc = mul2(f2(0.5f), f2(dd[h], dd[h + 1]));
+    const float2 dlim = mul2(f2(2.0f), f2(fminf(fabsf(dl[h]), fabsf(dr[h])), fminf(fabsf(dl[h + 1]), fabsf(dr[h + 1]))));
+    const float2 m = add2(f2(mR[h], mR[h + 1]), f2(mL[h], mL[h + 1]));
+    const float2 d4 = fma2(f2(4.0f / 3.0f), dc, mul2(f2(-1.0f / 6.0f), m));
+    const float2 pr = mul2(f2(dl[h], dl[h + 1]), f2(dr[h], dr[h + 1]));
+    const float mx = fminf(fabsf(d4.x), dlim.x), my = fminf(fabsf(d4.y), dlim.y);
+    const float2 d = mul2(f2(xi), f2(pr.x > 0.f ? copysignf(mx, d4.x) : 0.f, pr.y > 0.f ? copysignf(my, d4.y) : 0.f));
+    dq[h] = d.x;
+    dq[h + 1] = d.y;
   }
 }
 
