@@ -58,15 +58,15 @@ ALU_PEAK_SOURCE = {"fp32": "152 SMs x 128 FP32 lanes x 2 flops x 2070 MHz (unit 
 # algorithmic HBM bytes per zone-update of a fused step: one read and one write of the four conserved fields
 BYTES_PER_ZONE = {"fp32": 32, "fp64": 64}
 
-# The committed ncu summaries the DRAM traffic of a launch is read from: each names the kernel, the
-# workload, the command, the traffic per launch and the SHA-256 of the kernel's sources when captured.
+# The committed ncu summaries the DRAM traffic of a step's launches is read from: each names the kernels, the
+# workload, the command, the traffic and the SHA-256 of the kernel's sources when captured.
 # The figure is reported only while the sources still hash to it (else the counters describe another
 # kernel and traffic is null).
-TRAFFIC_PROFILES = {"sedov8192_learned": "profiles/ctu_step_fused_learned_fp32_sedov8192.md",
-                    "kh1024": "profiles/ctu_step_fused_fp32_kh1024.md"}
+TRAFFIC_PROFILES = {"sedov8192_learned": "profiles/march_step_fused_learned_fp32_sedov8192.md",
+                    "kh1024": "profiles/march_step_fused_fp32.md"}
 KERNEL_SOURCES = ["paper_1306_6883_gb300/csrc/" + f for f in
-                  ("k_ctu.cu", "ctu_kernels.cuh", "ctu_tile.cuh", "hydro_device.cuh", "mlp.cuh", "hydro_kernels.h",
-                   "tma.cuh")] + ["include/hydro.h"]
+                  ("k_ctu.cu", "ctu_kernels.cuh", "ctu_march.cuh", "march_kernels.cuh", "ctu_tile.cuh",
+                   "hydro_device.cuh", "soft_f64.cuh", "mlp.cuh", "hydro_kernels.h", "tma.cuh")]
 
 
 def kernel_sources_sha256():
@@ -78,7 +78,7 @@ def kernel_sources_sha256():
 
 
 def read_traffic(key):
-    """DRAM bytes per launch from a committed ncu summary: lines `traffic_bytes_per_launch: N` and
+    """DRAM bytes of one step's launches from a committed ncu summary: lines `traffic_bytes_per_launch: N` and
     `sources_sha256: H`.  Returns (bytes or None, note)."""
     path = TRAFFIC_PROFILES[key]
     try:
@@ -91,7 +91,7 @@ def read_traffic(key):
         return None, f"{path} holds no traffic figure"
     if h.group(1) != kernel_sources_sha256():
         return None, f"kernel sources changed since the capture in {path}"
-    return int(m.group(1)), f"ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch ({path})"
+    return int(m.group(1)), f"ncu dram__bytes_read.sum + dram__bytes_write.sum of one step's launches ({path})"
 
 
 def _peaks():

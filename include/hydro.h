@@ -200,8 +200,8 @@ hydro_status hydro_step_fused(hydro_ctx* ctx, double tmax);
  * graph for each pair of host buffers (and tmax) and replayed.  Returns when host_out holds the new state; the
  * context's current buffer holds it too.  The interior of host_out and of the current state equals what
  * hydro_upload, hydro_step_fused and hydro_download give; ghost cells are not filled (host_out's read as
- * 0 or as the values an earlier step left there).  Contexts with a learned model, a harvest or split = 1
- * run those three calls in turn.  The first call allocates two device copies of the state (unpitched,
+ * 0 or as the values an earlier step left there).  Contexts with a harvest or split = 1 run those three calls in
+ * turn.  The first call allocates two device copies of the state (unpitched,
  * 4 (nx + 2 ng)(ny + 2 ng) elements each), which the context keeps until hydro_destroy.
  * Errors: HYDRO_EINVAL (NULL pointers, host_in == host_out), HYDRO_ECUDA. */
 hydro_status hydro_step_host(hydro_ctx* ctx, const void* host_in, void* host_out, double tmax);

@@ -130,8 +130,9 @@ constexpr int F32_SMALL_TX = 16, F32_SMALL_TY = 8;
 constexpr int F64_TX = 16, F64_TY = 16, F64_NT = 384, F64_TY_SMALL = 8;
 
 // Resident blocks per SM the register allocator must allow: shared memory admits three tiles per SM in FP32
-// (three blocks of 384 threads need <= 56 registers) and in FP64 two of 16x16 (<= 85 registers); the small FP64
-// tile runs one to an SM.
+// (three blocks of 384 threads need <= 56 registers) and in FP64 two of 16x16 (<= 85 registers, at which the two-shock
+// step spills 64 bytes beside the arguments of its out-of-line solver: 0.9 % of the instructions of a KH 512^2 step are
+// local loads and stores); the small FP64 tile runs one to an SM.
 template <typename R, int TY>
 constexpr int min_blocks() {
   return is_f32<R>() ? HYDRO_F32_MINB : TY == F64_TY ? 2 : 1;

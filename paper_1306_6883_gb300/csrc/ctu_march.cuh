@@ -5,9 +5,9 @@
 // conversions, 1.2 times the tracing and the hat solves) and forms each MC slope three times and each shock detector
 // twice.  A strip loads, converts and traces a row once, keeps what it needs of the rows below in registers and rings
 // of rows, takes a column's own slopes and fluxes along y from the row before and a neighbour's along x from an
-// exchange row, and has no item arithmetic.  Sedov 4096^2, one step: 64.3 -> 40.9 warp instructions per zone, 1.09 ->
-// 0.75 ms (ncu); at 75 % issue with 16 warps an SM, where the tile had 79 % with 36.  The bound is still issue (ALU 42 %,
-// FMA pipe 47 %, shared memory 11 % of their rates).
+// exchange row, and has no item arithmetic.  Sedov 4096^2, one step: 64.3 -> 39.5 warp instructions per zone, 1.09 ->
+// 0.74 ms (ncu); at 74 % issue with 16 warps an SM, where the tile had 79 % with 36.  The bound is still issue (ALU 42 %,
+// FMA pipe 48 %, shared memory 11 % of their rates).  KH 1024^2, in segments of 16 rows: 52.2 and 69 %.
 //
 // What makes it so:
 //  - all threads of a block run all of every row's work, on copies of the edge columns outside the halo, so the loop
@@ -15,8 +15,10 @@
 //  - the two face solves of a stage run as a pair (riemann_pair), since four warps to a scheduler do not cover one
 //    solve's chain of dependent operations;
 //  - three barriers a row, with every exchange row written between one pair of them and read between the next;
-//  - 128 registers, no spills: four strips of 128 threads an SM (96 registers for five strips spilled: Sedov 4096^2
-//    1.22 ms; two threads a column, one for each direction, at 80 registers: KH 2048^2 317 us against 231).
+//  - 128 registers: four strips of 128 threads an SM.  The two-shock step spills nothing, HLLC and PPM 4 bytes, the learned
+//    one 12, ensembles (batch_march_kernel, whose members' parameters take registers) 36 to 48 (96 registers for five
+//    strips spilled 340: Sedov 4096^2 1.22 ms; two threads a column, one for each direction, at 80 registers: KH 2048^2
+//    317 us against 231).
 //
 // Row c is traced while row c + 3 arrives; the hat solves are row c's x faces and the y face c - 1/2 between the rows c -
 // 1 and c, the final ones the x faces of row c - 1 and the same y face, and the row updated is c - 1.  Results do not

@@ -53,7 +53,7 @@ struct TileLayout {
   static constexpr int SX = TX + 2, SY = TY + 2;  // cells whose face states are traced
   static constexpr int QP = QX;  // row pitch of the primitive tile
   // FP32 tiles keep the conserved values of the traced cells for the viscosity term (no global re-read);
-  // FP64 tiles re-read them from L2 to keep 3 CTAs per SM
+  // FP64 tiles re-read them from L2 to keep two CTAs per SM
   static constexpr bool SMEM_U = sizeof(R) == 4;
   static constexpr int nC = SX * SY;
   static constexpr int nQ = 4 * QP * QY;

@@ -6,8 +6,8 @@
 //  - along y a thread marches up a column, two rows at a time, the rows below in registers;
 //  - along x a warp takes 64 cells of a row, two a lane, 56 of them its own, and lanes exchange what their neighbours
 //    need by shuffles;
-// and the two faces of a thread are solved as a pair (riemann_pair).  485 and 541 instructions per zone, at 69 % of the
-// issue slots along x (20 warps an SM) and 55 % along y (the loop's chain: 12 to 16 warps).
+// and the two faces of a thread are solved as a pair (riemann_pair).  KH 1024^2: 490 and 575 instructions per zone, at
+// 68 % of the issue slots along x (20 warps an SM) and 61 % along y (16 warps; segments of 14 rows).
 #pragma once
 
 #include "ctu_march.cuh"
