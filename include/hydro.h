@@ -252,9 +252,8 @@ hydro_status hydro_conserved_totals_noalloc(const hydro_params* p, const void* d
  * upload a known state again (hydro_last_error says whether a copy was still outstanding when its tile
  * gave up, in which case later tiles on the same SM may have been overwritten as well).  Synchronises.
  * If stats is not NULL it receives {riemann solves, riemann iterations, unconverged solves} accumulated since
- * hydro_init.  They count the work done, which depends on how a step is cut: a face that two tiles or two strips solve
- * counts in each (the bands of host steps are strips of 4 or 16 rows), and so does what both launches of a learned
- * step solve; the FP32 sweeps of a split step count every face once. */
+ * hydro_init.  They count solves as the step is cut: a face that two tiles or two strips solve counts in each (the
+ * bands of host steps are strips of 4 or 16 rows); the FP32 sweeps of a split step count every face once. */
 hydro_status hydro_sync_status(hydro_ctx* ctx, unsigned long long stats[3]);
 
 /* Copy a host array into / out of the current state.  host has the dense layout

@@ -15,8 +15,8 @@
 //  - the two face solves of a stage run as a pair (riemann_pair), since four warps to a scheduler do not cover one
 //    solve's chain of dependent operations;
 //  - three barriers a row, with every exchange row written between one pair of them and read between the next;
-//  - 128 registers: four strips of 128 threads an SM.  The two-shock step spills nothing, HLLC and PPM 4 bytes, the learned
-//    one 12, ensembles (batch_march_kernel, whose members' parameters take registers) 36 to 48 (96 registers for five
+//  - 128 registers: four strips of 128 threads an SM.  The two-shock and the learned step spill nothing, HLLC and PPM 4
+//    bytes, ensembles (batch_march_kernel, whose members' parameters take registers) 36 to 48 (96 registers for five
 //    strips spilled 340: Sedov 4096^2 1.22 ms; two threads a column, one for each direction, at 80 registers: KH 2048^2
 //    317 us against 231).
 //
@@ -81,44 +81,66 @@ __device__ __forceinline__ void face_pair(const SP<float>& s, const float a[4], 
 
 // Work area of a learned step (learned_work_bytes, all zero between steps).  For each row of 32x16 tiles, four words of
 // which a launch uses those of its first row (the list's length, the next tile to take, the blocks that are done, -);
-// the list of the tiles to be stepped with the network, a band's part beginning at its first tile; and for each tile
-// what its cells are in the strips: status flags with LISTED, and FLT_MAX's bits less those of their least CFL value.
+// then for each tile what its cells are in the strips (count: solves in the high word, iterations past the first in the
+// low one; status flags with LISTED; FLT_MAX's bits less those of the least CFL value; solves that did not converge),
+// and the list of the tiles to be stepped with the network, a band's part beginning at its first tile.
 constexpr int LEARNED_TX = 32, LEARNED_TY = 16;
 struct LearnedWork {
   static constexpr unsigned int LISTED = 0x80000000u;
   unsigned int* counters;
+  unsigned long long* count;
+  unsigned int *state, *slack, *nonconv;
   int* list;
-  unsigned int *state, *slack;
   int tx;
   __device__ __forceinline__ LearnedWork(int nx, int ny, unsigned int* w, int by0) {
     tx = (nx + LEARNED_TX - 1) / LEARNED_TX;
     const int ty = (ny + LEARNED_TY - 1) / LEARNED_TY;
     const size_t n = (size_t)tx * ty;
     counters = w + 4 * (size_t)by0;
-    list = (int*)(w + 4 * (size_t)ty) + (size_t)by0 * tx;
-    state = w + 4 * (size_t)ty + n;
+    count = reinterpret_cast<unsigned long long*>(w + 4 * (size_t)ty);
+    state = reinterpret_cast<unsigned int*>(count + n);
     slack = state + n;
+    nonconv = slack + n;
+    list = reinterpret_cast<int*>(nonconv + n) + (size_t)by0 * tx;
   }
-  static constexpr size_t words(size_t tx, size_t ty) { return 4 * ty + 3 * tx * ty; }
+  static constexpr size_t words(size_t tx, size_t ty) { return 4 * ty + 6 * tx * ty; }
 };
 
 // What a strip's warp hands in for the tile row ty (counted over the grid of nx by ny cells) of its cells: the lanes'
-// status flags and least CFL value to the tiles of the columns col they belong to (at most two tiles, from left to
-// right), and to the list, each once, the tiles of the columns x - 1, x and x + 1 where left, own and right say so.
+// counts (at most 2^7 solves each, of maxiter iterations), status flags and least CFL value to the tiles of the columns
+// col they belong to (at most two tiles, from left to right), and to the list, each once, the tiles of the columns x - 1,
+// x and x + 1 where left, own and right say so.
 static __device__ __noinline__ void hand_in(int nx, int ny, unsigned int* work, int by0, int ty, int col, int x, bool left,
-                                            bool own, bool right, unsigned int flags, float cmin) {
+                                            bool own, bool right, TileCounters cnt, int maxiter, float cmin) {
   const LearnedWork w(nx, ny, work, by0);
   const int t = col / LEARNED_TX;
   const size_t row = (size_t)ty * w.tx;
   const int t0 = __shfl_sync(0xffffffffu, t, 0), t1 = __shfl_sync(0xffffffffu, t, 31);
+  const bool first = t == t0;
   const unsigned int slack = 0x7f7fffffu - __float_as_uint(cmin);
-  const unsigned int s0 = __reduce_max_sync(0xffffffffu, t == t0 ? slack : 0u);
-  const unsigned int s1 = __reduce_max_sync(0xffffffffu, t == t0 ? 0u : slack);
+  const unsigned int s0 = __reduce_max_sync(0xffffffffu, first ? slack : 0u);
+  const unsigned int s1 = __reduce_max_sync(0xffffffffu, first ? 0u : slack);
+  unsigned long long c0, c1;
+  if (maxiter < 256) {  // solves (a warp's in 12 bits) and iterations in one sum
+    const unsigned int c = cnt.solves | cnt.iters << 12;
+    const unsigned int p0 = __reduce_add_sync(0xffffffffu, first ? c : 0u);
+    const unsigned int p1 = __reduce_add_sync(0xffffffffu, first ? 0u : c);
+    c0 = (unsigned long long)(p0 & 0xfffu) << 32 | p0 >> 12;
+    c1 = (unsigned long long)(p1 & 0xfffu) << 32 | p1 >> 12;
+  } else {
+    c0 = (unsigned long long)__reduce_add_sync(0xffffffffu, first ? cnt.solves : 0u) << 32 |
+         __reduce_add_sync(0xffffffffu, first ? cnt.iters : 0u);
+    c1 = (unsigned long long)__reduce_add_sync(0xffffffffu, first ? 0u : cnt.solves) << 32 |
+         __reduce_add_sync(0xffffffffu, first ? 0u : cnt.iters);
+  }
   if ((threadIdx.x & 31) == 0) {
     if (s0) atomicMax(&w.slack[row + t0], s0);
     if (s1) atomicMax(&w.slack[row + t1], s1);
+    if (c0) atomicAdd(&w.count[row + t0], c0);
+    if (c1) atomicAdd(&w.count[row + t1], c1);
   }
-  if (flags) atomicOr(&w.state[row + t], flags);
+  if (cnt.flags) atomicOr(&w.state[row + t], cnt.flags);
+  if (cnt.nonconv) atomicAdd(&w.nonconv[row + t], cnt.nonconv);
   auto put = [&](int k) {
     if (!(atomicOr(&w.state[row + k], LearnedWork::LISTED) & LearnedWork::LISTED))
       w.list[atomicAdd(&w.counters[0], 1u)] = (int)row + k;
@@ -135,10 +157,11 @@ static __device__ __noinline__ void hand_in(int nx, int ny, unsigned int* work, 
 // one past the gate of mlp whose first iteration makes no small step (one of the cell's own faces, or a hat face that
 // corrects their states), go on the list of work, to be stepped with the network by a second launch, which overwrites
 // them; so the strip leaves a strong face after that iteration.  Every strip that has a cell solves all those faces, so
-// the list does not depend on how the grid is cut.  The cells' status flags and CFL values go to the tiles' records
-// (hand_in), of which the second launch takes those of the tiles that were not listed.  The network itself in the strip
-// would hold up all its later rows (a blast's front kept strips for 1 ms).  Strong faces are noted per column and
-// iteration c, as bit c mod 32 of a word for each of the four solves, and handed in at the end of each tile row.
+// the list does not depend on how the grid is cut.  What the strip counts, its status flags and CFL values go to the
+// tiles' records (hand_in), of which the second launch takes those of the tiles that were not listed.  The network
+// itself in the strip would hold up all its later rows (a blast's front kept strips for 1 ms).  Strong faces are noted
+// per column and iteration c, as bit c mod 32 of a word for each of the four solves, and handed in at the end of each
+// tile row (KH 3000^2: 448 us per plain step, 463 learned, 11 of them the second launch).
 template <int MODE, bool FUSED>
 __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, const StepFactors<float>& f,
                                           const float* __restrict__ Uin, float* __restrict__ Uout, int i0, int nv, int j0,
@@ -260,6 +283,7 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
     }
   };
   if constexpr (GATED) x_note[x] = x_note[W + x] = make_uint2(0, 0);
+  int c_in = j0;  // first row c whose solves have not been handed in
   int s3 = 0;  // ring slot of row c + 3
 #pragma unroll 1
   for (int c = j0 - 1; c <= j0 + nh; ++c) {
@@ -464,20 +488,25 @@ __device__ __forceinline__ void ctu_march(const KParams& P, const SP<float>& s, 
         x_note[W + x] = make_uint2(g.x & keep, g.y & keep);
         const bool hy = (h.y & bits(r0)) != 0, mine = (g.x & bits(r0)) != 0;
         const bool both = ((h.x & bits(r0 - 1)) | (g.y & bits(r0 + 1))) != 0 || hy;
-        const int k = x < 4 ? 0 : x > nv + 3 ? nv - 1 : x - 4;  // the strip's column
+        // a row c from j0 on has on_xface twice, on_trace and on_cell; row j0 - 1's x faces make up for row j0's
+        cnt.solves = (unsigned int)(c + 1 - c_in) * ((on_xface ? 2 : 0) + (on_trace ? 1 : 0) + (on_cell ? 1 : 0));
+        const int k = x < 4 ? 0 : x > nv + 3 ? nv - 1 : x - 4;  // the strip's column this thread's faces belong to
         hand_in(P.nx, P.ny, work, by0, (c - 1 - P.ng) / LEARNED_TY, i0 - P.ng + k, i0 - P.ng + x - 4,
-                both && x >= 5 && x <= nv + 4, (both || mine) && on_cell, hy && x >= 3 && x <= nv + 2, cnt.flags,
+                both && x >= 5 && x <= nv + 4, (both || mine) && on_cell, hy && x >= 3 && x <= nv + 2, cnt, s.maxiter,
                 FUSED ? *cfl_min : FLT_MAX);
-        cnt.flags = 0;
+        cnt = TileCounters();
         if constexpr (FUSED) *cfl_min = FLT_MAX;
+        c_in = c + 1;
       }
     }
     s3 = s3 + 1 == MARCH_ROWS ? 0 : s3 + 1;
   }
   // every face above counted once; the iterations past the first were added as they ran
-  const unsigned int solves = (on_xface ? 2 * nh + 2 : 0) + (on_trace ? nh + 1 : 0) + (on_cell ? nh + 1 : 0);
-  cnt.solves += solves;
-  if (face_kind(MODE) != FACE_HLLC) cnt.iters += solves;
+  if constexpr (!GATED) {
+    const unsigned int solves = (on_xface ? 2 * nh + 2 : 0) + (on_trace ? nh + 1 : 0) + (on_cell ? nh + 1 : 0);
+    cnt.solves += solves;
+    if (face_kind(MODE) != FACE_HLLC) cnt.iters += solves;
+  }
 }
 
 }  // namespace hydro

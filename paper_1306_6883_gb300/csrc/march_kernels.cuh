@@ -113,10 +113,15 @@ __global__ void __launch_bounds__(320, 2)
   for (int k = first + blockIdx.x * blockDim.x + threadIdx.x; k < first + tiles; k += gridDim.x * blockDim.x) {
     const unsigned int state = w.state[k];
     if (!(state & LearnedWork::LISTED)) {
+      const unsigned long long c = w.count[k];
       cnt.flags |= state;
+      cnt.solves += (unsigned int)(c >> 32);
+      cnt.iters += (unsigned int)(c >> 32) + (unsigned int)c;
+      cnt.nonconv += w.nonconv[k];
       cmin = fminf(cmin, __uint_as_float(0x7f7fffffu - w.slack[k]));
     }
-    w.state[k] = w.slack[k] = 0u;
+    w.state[k] = w.slack[k] = w.nonconv[k] = 0u;
+    w.count[k] = 0ull;
   }
   flush_counters(cnt, scr);
   if constexpr (FUSED)

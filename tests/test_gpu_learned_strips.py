@@ -108,3 +108,23 @@ def test_no_cell_keeps_what_a_strip_left_unsolved(torch, gate, fused):
     a.close()
     b.close()
     m.close()
+
+
+def test_a_cell_stepped_by_both_launches_counts_once(torch):
+    # the blast lists half a percent of the tiles; a tile solves a tenth more faces per cell than a strip
+    from paper_1306_6883_gb300 import hydro as H
+    from paper_1306_6883_gb300.solver import Model, Solver, params_for
+    pr, U = _evolved(torch, 2100, 1800)
+    m = Model(seed=3)
+    counts = []
+    for learned, gate in ((0, None), (1, (40.0, 1e9)), (1, (0.35, 1.0))):
+        s = Solver(params_for(pr, H.HYDRO_FP32, use_learned_guess=learned), U)
+        if learned:
+            m.set_gate(*gate)
+            H.hydro_set_riemann_model(s.ctx, m.m)
+        s.step_fused()
+        counts.append(s.status()[1])
+        s.close()
+    assert counts[0] == counts[1]  # nothing listed
+    assert counts[0][0] < counts[2][0] < 1.001 * counts[0][0]
+    m.close()
