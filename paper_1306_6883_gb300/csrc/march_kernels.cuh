@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(MARCH_MAX_THREADS, MARCH_SM_THREADS / MARCH_MA
 // until it is empty), which overwrite the strips' cells; the records of the tiles that were not listed; and for a fused
 // step its end.  by0, rows: the tile rows of the launch (a band of the step, or all).  Bound by the chain of stages of
 // the few tiles it has (11 us without any, 38 with those of a blast's front; ncu).  Sedov 8192^2 learned, one step: 4.73 ms
-// with all tiles in the tile kernel, 3.13 in strips with this launch (3.40 when a strip tested every face's gate and
+// with all tiles in the tile kernel, 3.07 in strips with this launch (3.40 when a strip tested every face's gate and
 // gave up at the first strong one, and the list depended on the cut); with the network called from the strip's loop the
 // strips on the blast's front took 1 ms each.
 // Two blocks an SM: with three the registers (64) spilled 136 bytes in the chain (Sedov 3000^2 503 us per step, 488 with
