@@ -657,7 +657,7 @@ def kh_line(flush, steps, warmup):
     a32, a64 = arm_summary(pr, r32), arm_summary(pr, r64)
     kern = sum(r32["step_ms"]) / len(r32["step_ms"])
     return {"workload": wname, "fp32": a32, "fp64": a64, "fp32_speedup_over_fp64": a32["value"] / a64["value"],
-            "roofline_fp32": roofline("fp32", zones, kern, r32["iters_per_solve"], "ctu_step_fused_kernel", "kh1024"),
+            "roofline_fp32": roofline("fp32", zones, kern, r32["iters_per_solve"], "march_step_fused_kernel<FACE_PLAIN>", "kh1024"),
             "l2": "flushed (256 MB write) before every timed step"}
 
 
@@ -671,7 +671,7 @@ def sedov4096_line(model, steps, warmup, world):
         r = run_arm(pr, prec, steps, warmup, model=m, keep_state=False)
         a = arm_summary(pr, r)
         kern = sum(r["step_ms"]) / len(r["step_ms"])
-        rl = roofline(prec, zones, kern, r["iters_per_solve"], "ctu_step_fused_kernel")
+        rl = roofline(prec, zones, kern, r["iters_per_solve"], "march_step_fused_kernel<FACE_PLAIN>")
         arms[name] = dict(a, roofline_frac=rl["frac"], hbm_frac=rl["hbm"]["frac"])
     out = {"workload": wname, "steps": steps, "arms": arms,
            "speedup_fp32_learned_over_fp64": arms["fp32_learned"]["value"] / arms["fp64_plain"]["value"],
