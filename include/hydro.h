@@ -275,7 +275,9 @@ hydro_status hydro_download(hydro_ctx* ctx, void* host);
  * activations, FP32 accumulation), 32 faces per warp; a warp evaluates the network only when one of its
  * faces has |ln(p_L/p_R)|/2 > gate_dp or |u_L - u_R|/c_ref > gate_du, otherwise its faces start from the
  * acoustic estimate.  Large grids step in strips from the acoustic estimate, and from the network only the 32x16
- * tiles with a cell whose update reads a face past the gate that one iteration does not solve. */
+ * tiles with a cell whose update reads a face past the gate that one iteration does not solve.  A tile queues at most
+ * 128 faces for the network in each of its two solve stages; of more, those that start from the acoustic estimate are
+ * not always the same, so steps with such tiles repeat to rounding, not bit for bit. */
 typedef struct hydro_mlp hydro_mlp;
 
 /* Create a network with He-normal weights drawn from `seed` (counter-based generator on the device).
